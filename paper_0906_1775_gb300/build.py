@@ -43,7 +43,7 @@ def flags(extra=()):
 def _stale(obj: str, src: str) -> bool:
     if not os.path.exists(obj):
         return True
-    deps = [src, os.path.join(CSRC, "internal.cuh"), os.path.join(CSRC, "operator_kernels.cuh"),
+    deps = [src, os.path.join(CSRC, "internal.cuh"), os.path.join(CSRC, "operator_kernels.cuh"), os.path.join(CSRC, "operator_reg.cuh"),
             os.path.join(INCLUDE, "madmap.h")]
     return any(os.path.getmtime(d) > os.path.getmtime(obj) for d in deps)
 

@@ -252,6 +252,25 @@ __device__ __forceinline__ int otf_row(const OtfPointing& o, long long t, bool p
   return g >= 0 ? o.g2o[g] : -1;
 }
 
+// Twiddles of the float32 register transforms (operator_reg.cuh), M = 256 N1:
+// per index i the powers 1, 2, 4, 8, 16 of w_i (pairs (w, w^2), (w^4, w^8),
+// (w^16, 0)), and the four-step twiddles of the first 16 spectral rows.
+struct RegTables {
+  int logN1 = 0;                  // 0: the length has no register transform
+  const float4* col = nullptr;    // [16][2]  w_j = exp(-2 pi i j / 256)
+  const float4* row = nullptr;    // [32][4]  w_l = exp(-2 pi i l / N1) (last entry 0)
+  const float4* four = nullptr;   // [N1][2]  w_n1 = exp(-2 pi i 16 n1 / M)
+  const float2* four0 = nullptr;  // [16][N1] exp(-2 pi i n1 p / M)
+};
+constexpr int REG_N2 = 256;       // column length of the register transforms
+// log2(N1) of the register transforms of length M, or 0.
+inline int reg_log_n1(int M) { return (M >= (1 << 14) && M <= (1 << 18)) ? __builtin_ctz((unsigned)M) - 8 : 0; }
+// The tables of one length as one array (the order of the struct's pointers).
+size_t reg_table_floats(int logN1);
+void reg_fill_tables(int logN1, float* out);
+RegTables reg_point_tables(int logN1, const float* base);
+void reg_spectrum(const std::vector<double>& re, int logN1, float* h32);
+
 // ---------------------------------------------------------------- plan
 struct SolveBuffers;  // solver.cu
 
@@ -280,9 +299,10 @@ struct Plan {
   float* P32 = nullptr;            // [n_obs][8] (IQU) or [n_obs] (T)
   Tile* tiles = nullptr;           // [n_tiles]
   double* H64 = nullptr;           // [n_filters][M] permuted spectra / M
-  float* H32 = nullptr;
+  float* H32 = nullptr;            // as H64, or [k2][k1] natural order for register transforms
   double2* tw64 = nullptr;         // [M] exp(-2 pi i j / M)
-  float2* tw32 = nullptr;
+  float2* tw32 = nullptr;          // (NULL with register transforms)
+  RegTables reg;                   // float32 register transforms
   df64* Hdf = nullptr;             // [n_filters][M] H64 as double-float pairs
   cdf64* twdf = nullptr;           // [M] tw64 as double-float pairs
   float4* csdf = nullptr;          // [n_t] cs64 as double-float pairs (IQU)
@@ -425,15 +445,10 @@ madmap_status op_launch(Plan* p, int prec, int in_mode, int out_mode, const void
                         long long in_stride, long long out_stride, int n_rhs, const int* skip,
                         cudaStream_t s);
 
-size_t f1_smem_bytes(const Plan* p, int prec);
-
 // Event timing of the map-to-map operator: ms[0..2] mean duration of one
 // launch of each kernel (chunks run one after another on `s`), ms[3] mean
 // duration of one application as the solver launches it.
 madmap_status op_time(Plan* p, int prec, const void* in, void* out, int reps, double ms[4], cudaStream_t s);
-
-// Resident CTAs per SM of the operator kernels and CTAs per tile.
-void op_occupancy(const Plan* p, int prec, int& ctas_per_sm, int& ctas_per_tile);
 
 // Number of operator launches per application and tiles per launch.
 void chunking(const Plan* p, int& n_chunks, int& per_chunk, int n_tiles = -1);
@@ -457,8 +472,6 @@ struct OpImpl {
                               long long out_stride, const int* skip, int skip_stride, const TileSet* ts,
                               cudaStream_t s);
   madmap_status (*time)(Plan* p, const void* in, void* out, int reps, double ms[4], cudaStream_t s);
-  void (*occupancy)(const Plan* p, int& ctas_per_sm, int& ctas_per_tile);  // NULL for double-float
-  size_t (*f13_smem)(const Plan* p);
   // the (cos 2psi, sin 2psi) weights of n angles as this precision's kernels form them
   madmap_status (*weights)(long long n, const float* psi, void* c, void* s, cudaStream_t st);
 };

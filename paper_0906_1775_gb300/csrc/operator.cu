@@ -70,13 +70,6 @@ madmap_status op_time(Plan* p, int prec, const void* in, void* out, int reps, do
   return impl_for(prec).time(p, in, out, reps, ms, s);
 }
 
-// The float64 kernels' occupancy stands for the double-float ones too.
-void op_occupancy(const Plan* p, int prec, int& ctas_per_sm, int& ctas_per_tile) {
-  (prec == OPP_F32 ? op_impl_f32() : op_impl_f64()).occupancy(p, ctas_per_sm, ctas_per_tile);
-}
-
-size_t f1_smem_bytes(const Plan* p, int prec) { return impl_for(prec).f13_smem(p); }
-
 // in_mode: IN_MAP (gather from a map), IN_TOD (float timestream, e.g. the
 // data d) or IN_TOD_REAL (timestream of the working precision).  n_rhs == 0
 // only prepares the kernels (shared-memory opt-in) and launches nothing.
@@ -203,8 +196,10 @@ extern "C" madmap_status madmap_apply_ninv_noalloc(int32_t precision, int64_t n_
   build_tiles(off, filt, n_filters, n_lags, M, tiles);
   q.n_tiles = (int)tiles.size();
   const size_t ce = fp64 ? sizeof(double2) : sizeof(float2), re = fp64 ? sizeof(double) : sizeof(float);
+  const int rl = fp64 ? 0 : reg_log_n1(M);   // register transforms: their tables take the twiddles' place
+  const size_t tw_bytes = rl > 0 ? sizeof(float) * reg_table_floats(rl) : (size_t)M * ce;
   const size_t off_tw = 0;
-  const size_t off_H = align256(off_tw + (size_t)M * ce);
+  const size_t off_H = align256(off_tw + tw_bytes);
   const size_t off_T = align256(off_H + (size_t)n_filters * M * re);
   const size_t off_S = align256(off_T + tiles.size() * sizeof(Tile));
   const size_t per_tile = (size_t)M * ce;
@@ -213,7 +208,8 @@ extern "C" madmap_status madmap_apply_ninv_noalloc(int32_t precision, int64_t n_
   const long long cap = (long long)(((size_t)MADMAP_NOALLOC_SCRATCH_BYTES - off_S) / per_tile);
   q.tiles_per_chunk = (int)std::max(1LL, std::min<long long>(std::min<long long>(cap, 65535), std::max(1, q.n_tiles)));
   // host-side tables: twiddles exp(-2 pi i j / M) and the permuted circulant spectra / M
-  std::vector<double> h64((size_t)n_filters * M);
+  std::vector<double> h64(rl > 0 ? 0 : (size_t)n_filters * M);
+  std::vector<float> h32(fp64 ? 0 : (size_t)n_filters * M);
   std::vector<double> re_(M), im_(M);
   for (int f = 0; f < n_filters; ++f) {
     std::fill(re_.begin(), re_.end(), 0.0);
@@ -228,6 +224,10 @@ extern "C" madmap_status madmap_apply_ninv_noalloc(int32_t precision, int64_t n_
     double mn = 1e300;
     for (int k = 0; k < M; ++k) mn = std::min(mn, re_[k]);
     MM_CHECK(mn > 0.0, MADMAP_ERR_NOT_PD, "apply_ninv_noalloc: a filter is not positive definite");
+    if (rl > 0) {
+      reg_spectrum(re_, rl, h32.data() + (size_t)f * M);
+      continue;
+    }
     for (int p2 = 0; p2 < q.N2; ++p2) {
       int k2 = 0;
       for (int b = 0; b < q.logN2; ++b) k2 |= ((p2 >> b) & 1) << (q.logN2 - 1 - b);
@@ -253,16 +253,21 @@ extern "C" madmap_status madmap_apply_ninv_noalloc(int32_t precision, int64_t n_
     q.tw64 = reinterpret_cast<double2*>(b + off_tw);
     q.H64 = reinterpret_cast<double*>(b + off_H);
   } else {
-    std::vector<float2> t32(M);
-    std::vector<float> h32(h64.size());
-    for (int j = 0; j < M; ++j) {
-      const double ang = 2.0 * M_PI * (double)j / (double)M;
-      t32[j] = make_float2((float)cos(ang), (float)-sin(ang));
+    std::vector<float> t32(tw_bytes / sizeof(float));
+    if (rl > 0) {
+      reg_fill_tables(rl, t32.data());
+      q.reg = reg_point_tables(rl, reinterpret_cast<const float*>(b + off_tw));
+    } else {
+      for (int j = 0; j < M; ++j) {
+        const double ang = 2.0 * M_PI * (double)j / (double)M;
+        t32[2 * j] = (float)cos(ang);
+        t32[2 * j + 1] = (float)-sin(ang);
+      }
+      q.tw32 = reinterpret_cast<float2*>(b + off_tw);
     }
     for (size_t k = 0; k < h64.size(); ++k) h32[k] = (float)h64[k];
-    MM_CUDA(cudaMemcpyAsync(b + off_tw, t32.data(), (size_t)M * sizeof(float2), cudaMemcpyHostToDevice, s));
+    MM_CUDA(cudaMemcpyAsync(b + off_tw, t32.data(), tw_bytes, cudaMemcpyHostToDevice, s));
     MM_CUDA(cudaMemcpyAsync(b + off_H, h32.data(), h32.size() * sizeof(float), cudaMemcpyHostToDevice, s));
-    q.tw32 = reinterpret_cast<float2*>(b + off_tw);
     q.H32 = reinterpret_cast<float*>(b + off_H);
   }
   if (!tiles.empty())

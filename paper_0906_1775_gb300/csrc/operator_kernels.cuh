@@ -104,6 +104,11 @@ struct OpArgs {
   void* scratch;
   const void* H;
   const void* tw;
+  // float32 register transforms (operator_reg.cuh): log2 of the row length, and
+  // twiddle tables (RegTables)
+  int reg_logN1;
+  const float4 *reg_col, *reg_row, *reg_four;
+  const float2* reg_four0;
   int n_rep;          // > 1: map outputs go to replica (blockIdx.x + blockIdx.y) % n_rep, rep_stride apart
   int runs;           // scatter runs of consecutive samples that hit one pixel with one atomic (run_*)
   long long rep_stride;
@@ -599,6 +604,196 @@ __device__ __forceinline__ T run_sum(T x, int start) {
   return x;
 }
 
+// ---------------------------------------------------------------- gather and scatter of a batch
+// The input values of window positions nn[0 .. U-1] of both lanes (positions
+// outside a lane, and nn < 0, give 0), all loads of the batch issued before
+// any is consumed.
+template <typename Real, int NS, int IN, int U>
+__device__ __forceinline__ void gather_samples(const OpArgs& a, const LaneView<Real> (&L)[2], const int (&nn)[U],
+                                               Real (&v)[2][U]) {
+  bool ok[2][U];
+#pragma unroll
+  for (int u = 0; u < U; ++u)
+#pragma unroll
+    for (int l = 0; l < 2; ++l) ok[l][u] = in_range(nn[u], L[l].in_lo, L[l].in_hi);
+  if (!gathers(IN)) {
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int l = 0; l < 2; ++l) {
+        if (IN == IN_TODF)
+          v[l][u] = ok[l][u] ? (Real)__ldg(static_cast<const float*>(L[l].in) + nn[u]) : Real(0);
+        else
+          v[l][u] = ok[l][u] ? static_cast<const Real*>(L[l].in)[nn[u]] : Real(0);
+      }
+  } else {
+    int pp[2][U], qq[2][U];
+    Real cc[2][U], ss[2][U];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int l = 0; l < 2; ++l) {
+        load_pointing<Real, NS>(a, L[l], nn[u], ok[l][u], pp[l][u], cc[l][u], ss[l][u]);
+        if constexpr (NS == NS_MR || extended(NS)) {
+          const int* qp = NS == NS_MR ? L[l].pq : L[l].pe;
+          qq[l][u] = (ok[l][u] && qp) ? __ldg(qp + nn[u]) : -1;
+        }
+      }
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int l = 0; l < 2; ++l) {
+        Real c = cc[l][u], sn = ss[l][u];
+        if (polarised(NS) && !on_the_fly(NS)) finish_angle<Real>(c, sn);
+        const Real* x = static_cast<const Real*>(L[l].in);
+        if constexpr (NS == NS_MR) {
+          v[l][u] = pp[l][u] >= 0 ? gather_mr<Real>(x, pp[l][u], qq[l][u], c, sn) : Real(0);
+        } else {
+          v[l][u] = pp[l][u] >= 0 ? gather<Real, map_ns(NS)>(x, pp[l][u], c, sn) : Real(0);
+          if constexpr (extended(NS)) {   // + the extra column's amplitude (slot 0 of its row)
+            if (pp[l][u] >= 0 && qq[l][u] >= 0) v[l][u] += x[(long long)qq[l][u] * (map_ns(NS) == 3 ? 4 : 1)];
+            if (pp[l][u] >= 0 && L[l].hb) {   // + the half-wave-plate term
+              const int hb = __ldg(L[l].hb + nn[u]);
+              if (hb >= 0)
+                v[l][u] += hwp_gather<Real>(x, hb, map_ns(NS) == 3 ? 4 : 1, __ldg(L[l].hang + nn[u]),
+                                            __ldg(L[l].htau + nn[u]));
+            }
+          }
+        }
+      }
+  }
+  if constexpr (IN == IN_RESX) {   // d - A x (flagged samples: rows of A are zero)
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int l = 0; l < 2; ++l)
+        if (ok[l][u]) v[l][u] = Real(__ldg(L[l].in2 + nn[u])) - v[l][u];
+  }
+}
+
+// The outputs of window positions nn[0 .. U-1] with values val (lane 0, lane 1).
+// RUNB > 0: the warp's lanes hold groups of RUNB consecutive samples.  hacc,
+// hgrp: the CTA's half-wave-plate sums (extended pointing only).
+template <typename Real, int NS, int OUT, int U, int RUNB>
+__device__ __forceinline__ void scatter_samples(const OpArgs& a, const LaneView<Real> (&L)[2], const int (&nn)[U],
+                                                const Real (&val)[2][U], typename OutT<Real>::type* hacc, int* hgrp) {
+  bool ok[2][U];
+#pragma unroll
+  for (int u = 0; u < U; ++u)
+#pragma unroll
+    for (int l = 0; l < 2; ++l) ok[l][u] = in_range(nn[u], L[l].out_lo, L[l].out_hi);
+  if (OUT == OUT_TOD) {
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int l = 0; l < 2; ++l)
+        if (ok[l][u]) static_cast<typename OutT<Real>::type*>(L[l].out)[nn[u]] = to_out(val[l][u]);
+  } else if constexpr (std::is_same<Real, df64>::value && polarised(NS)) {
+    // double-float: round the value to float64 once and weight it with the
+    // float64 (cos, sin) pair (5 float64 operations per sample, not 9)
+    int pp[2][U], qq[2][U], ee[2][U];
+    double2 cs[2][U];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int l = 0; l < 2; ++l) {
+        if constexpr (on_the_fly(NS)) {
+          df64 c, sn;
+          load_pointing<Real, NS>(a, L[l], nn[u], ok[l][u], pp[l][u], c, sn);
+          cs[l][u] = make_double2(to_double(c), to_double(sn));
+        } else {
+          pp[l][u] = ok[l][u] ? __ldg(L[l].pix + nn[u]) : -1;
+          cs[l][u] = ok[l][u] ? L[l].cs[nn[u]] : make_double2(0.0, 0.0);
+        }
+        if constexpr (NS == NS_MR) qq[l][u] = ok[l][u] ? __ldg(L[l].pq + nn[u]) : -1;
+        else qq[l][u] = pp[l][u];
+        if constexpr (extended(NS)) ee[l][u] = (ok[l][u] && L[l].pe) ? __ldg(L[l].pe + nn[u]) : -1;
+      }
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int l = 0; l < 2; ++l) {
+        if (pp[l][u] < 0) continue;
+        double* y = static_cast<double*>(L[l].out);
+        const double v = to_double(val[l][u]);
+        atomicAdd(y + 4LL * pp[l][u], v);
+        atomicAdd(y + 4LL * qq[l][u] + 1, v * cs[l][u].x);
+        atomicAdd(y + 4LL * qq[l][u] + 2, v * cs[l][u].y);
+        if constexpr (extended(NS)) {
+          if (ee[l][u] >= 0) atomic_add_warp(y, 4LL * ee[l][u], v);
+        }
+      }
+  } else {
+    int pp[2][U], qq[2][U];
+    Real cc[2][U], ss[2][U];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int l = 0; l < 2; ++l) {
+        load_pointing<Real, NS>(a, L[l], nn[u], ok[l][u], pp[l][u], cc[l][u], ss[l][u]);
+        if constexpr (NS == NS_MR || extended(NS)) {
+          const int* qp = NS == NS_MR ? L[l].pq : L[l].pe;
+          qq[l][u] = (ok[l][u] && qp) ? __ldg(qp + nn[u]) : -1;
+        }
+      }
+    // float32: one atomic per run of samples in one pixel (in float64 and
+    // double-float the shuffles of the partial sums cost more than the
+    // atomics they save)
+    if constexpr (RUNB > 0 && (NS == 1 || NS == 3) && std::is_same<Real, float>::value) {
+      if (a.runs) {
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+          for (int l = 0; l < 2; ++l) {
+            int start;
+            bool tail;
+            run_geometry<RUNB>(pp[l][u], start, tail);
+            const float v = pp[l][u] >= 0 ? val[l][u] : 0.0f;
+            const float s0 = run_sum<RUNB>(v, start);
+            if constexpr (NS == 1) {
+              if (tail && pp[l][u] >= 0) atomicAdd(static_cast<float*>(L[l].out) + pp[l][u], s0);
+            } else {
+              float c = cc[l][u], sn = ss[l][u];
+              finish_angle<float>(c, sn);
+              const float s1 = run_sum<RUNB>(v * c, start), s2 = run_sum<RUNB>(v * sn, start);
+              if (tail && pp[l][u] >= 0)
+                atomicAdd(reinterpret_cast<float4*>(L[l].out) + pp[l][u], make_float4(s0, s1, s2, 0.0f));
+            }
+          }
+        return;
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int l = 0; l < 2; ++l) {
+        if (pp[l][u] < 0) continue;
+        if constexpr (extended(NS)) {   // the extra column's share (slot 0 of its row)
+          typedef typename OutT<Real>::type Out;
+          if (qq[l][u] >= 0)
+            atomic_add_warp(static_cast<Out*>(L[l].out), (long long)qq[l][u] * (map_ns(NS) == 3 ? 4 : 1),
+                            (Out)to_out(val[l][u]));
+        }
+        Real c = cc[l][u], sn = ss[l][u];
+        if (polarised(NS) && !on_the_fly(NS)) finish_angle<Real>(c, sn);
+        if constexpr (NS == NS_MR)
+          scatter_mr<Real>(static_cast<typename OutT<Real>::type*>(L[l].out), pp[l][u], qq[l][u], val[l][u], c, sn);
+        else
+          scatter<Real, map_ns(NS)>(static_cast<typename OutT<Real>::type*>(L[l].out), pp[l][u], val[l][u], c, sn);
+      }
+  }
+  if constexpr (extended(NS) && OUT == OUT_MAP) {
+    if (a.hwp_base) {   // half-wave-plate parameters, one converged warp at a time
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int l = 0; l < 2; ++l)
+          hwp_scatter_warp<Real>(hacc + 32 * l, hgrp + l, L[l].pix, L[l].hb, L[l].hang, L[l].htau, nn[u],
+                                 ok[l][u], val[l][u]);
+    }
+  }
+}
+
 // ---------------------------------------------------------------- k_f1
 // LG2 > 0 fixes the column length N2 = 2^LG2 at compile time (and with it the
 // CTA's column count); LG2 = 0 reads the geometry from the arguments.
@@ -630,72 +825,8 @@ __global__ void __launch_bounds__(256, sizeof(Real) == 4 ? MM_MINB_F13 : MM_MINB
   const int total = B1 << logN2;
   constexpr int bd = OP_THREADS;
   constexpr int U = (gathers(IN) && polarised(NS)) ? MM_U_GATHER : 8;
-  // the input values of elements ee[0 .. U-1] (lane 0, lane 1), all loads of
-  // the batch issued before any is consumed
-  auto gather_batch = [&](const int (&ee)[U], Real (&v)[2][U]) {
-    int nn[U];
-    bool ok[2][U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int e = ee[u];
-      nn[u] = n1_0 + (e & (B1 - 1)) + ((e >> logB1) << a.logN1);
-#pragma unroll
-      for (int l = 0; l < 2; ++l) ok[l][u] = e < total && in_range(nn[u], L[l].in_lo, L[l].in_hi);
-    }
-    if (!gathers(IN)) {
-#pragma unroll
-      for (int u = 0; u < U; ++u)
-#pragma unroll
-        for (int l = 0; l < 2; ++l) {
-          if (IN == IN_TODF)
-            v[l][u] = ok[l][u] ? (Real)__ldg(static_cast<const float*>(L[l].in) + nn[u]) : Real(0);
-          else
-            v[l][u] = ok[l][u] ? static_cast<const Real*>(L[l].in)[nn[u]] : Real(0);
-        }
-    } else {
-      int pp[2][U], qq[2][U];
-      Real cc[2][U], ss[2][U];
-#pragma unroll
-      for (int u = 0; u < U; ++u)
-#pragma unroll
-        for (int l = 0; l < 2; ++l) {
-          load_pointing<Real, NS>(a, L[l], nn[u], ok[l][u], pp[l][u], cc[l][u], ss[l][u]);
-          if constexpr (NS == NS_MR || extended(NS)) {
-            const int* qp = NS == NS_MR ? L[l].pq : L[l].pe;
-            qq[l][u] = (ok[l][u] && qp) ? __ldg(qp + nn[u]) : -1;
-          }
-        }
-#pragma unroll
-      for (int u = 0; u < U; ++u)
-#pragma unroll
-        for (int l = 0; l < 2; ++l) {
-          Real c = cc[l][u], sn = ss[l][u];
-          if (polarised(NS) && !on_the_fly(NS)) finish_angle<Real>(c, sn);
-          const Real* x = static_cast<const Real*>(L[l].in);
-          if constexpr (NS == NS_MR) {
-            v[l][u] = pp[l][u] >= 0 ? gather_mr<Real>(x, pp[l][u], qq[l][u], c, sn) : Real(0);
-          } else {
-            v[l][u] = pp[l][u] >= 0 ? gather<Real, map_ns(NS)>(x, pp[l][u], c, sn) : Real(0);
-            if constexpr (extended(NS)) {   // + the extra column's amplitude (slot 0 of its row)
-              if (pp[l][u] >= 0 && qq[l][u] >= 0) v[l][u] += x[(long long)qq[l][u] * (map_ns(NS) == 3 ? 4 : 1)];
-              if (pp[l][u] >= 0 && L[l].hb) {   // + the half-wave-plate term
-                const int hb = __ldg(L[l].hb + nn[u]);
-                if (hb >= 0)
-                  v[l][u] += hwp_gather<Real>(x, hb, map_ns(NS) == 3 ? 4 : 1, __ldg(L[l].hang + nn[u]),
-                                              __ldg(L[l].htau + nn[u]));
-              }
-            }
-          }
-        }
-    }
-    if constexpr (IN == IN_RESX) {   // d - A x (flagged samples: rows of A are zero)
-#pragma unroll
-      for (int u = 0; u < U; ++u)
-#pragma unroll
-        for (int l = 0; l < 2; ++l)
-          if (ok[l][u]) v[l][u] = Real(__ldg(L[l].in2 + nn[u])) - v[l][u];
-    }
-  };
+  // window position of CTA element e (-1 past the CTA's elements)
+  auto position = [&](int e) { return e < total ? n1_0 + (e & (B1 - 1)) + ((e >> logB1) << a.logN1) : -1; };
   // float32 with compile-time geometry: thread t's 16 elements t + 256 u are
   // the two radix-8 groups (bases p0 and p0 + N2/16, stride N2/8) of the first
   // column pass, which therefore runs in registers before the first store
@@ -710,11 +841,11 @@ __global__ void __launch_bounds__(256, sizeof(Real) == 4 ? MM_MINB_F13 : MM_MINB
       C gv[8];
 #pragma unroll
       for (int b = 0; b < 8 / U; ++b) {
-        int ee[U];
+        int nn[U];
         Real v[2][U];
 #pragma unroll
-        for (int k = 0; k < U; ++k) ee[k] = threadIdx.x + (2 * (U * b + k) + G) * bd;
-        gather_batch(ee, v);
+        for (int k = 0; k < U; ++k) nn[k] = position(threadIdx.x + (2 * (U * b + k) + G) * bd);
+        gather_samples<Real, NS, IN, U>(a, L, nn, v);
 #pragma unroll
         for (int k = 0; k < U; ++k) {
           gv[U * b + k].x = v[0][k];
@@ -728,14 +859,14 @@ __global__ void __launch_bounds__(256, sizeof(Real) == 4 ? MM_MINB_F13 : MM_MINB
     }
   } else {
     for (int e0 = threadIdx.x; e0 < total; e0 += bd * U) {
-      int ee[U];
+      int nn[U];
       Real v[2][U];
 #pragma unroll
-      for (int u = 0; u < U; ++u) ee[u] = e0 + u * bd;
-      gather_batch(ee, v);
+      for (int u = 0; u < U; ++u) nn[u] = position(e0 + u * bd);
+      gather_samples<Real, NS, IN, U>(a, L, nn, v);
 #pragma unroll
       for (int u = 0; u < U; ++u) {
-        const int e = ee[u];
+        const int e = e0 + u * bd;
         if (e < total) {
           C z;
           z.x = v[0][u];
@@ -957,128 +1088,7 @@ __global__ void __launch_bounds__(256, sizeof(Real) == 4 ? MM_MINB_F13 : MM_MINB
   constexpr int U = OUT == OUT_MAP ? MM_U_SCATTER : 8;
   // lanes per group of consecutive samples (compile-time geometry only)
   constexpr int RUNB = LG2 > 0 ? ((1 << (ELOG - LG2)) < 32 ? (1 << (ELOG - LG2)) : 32) : 0;
-  // the outputs of elements ee[0 .. U-1] with values val (lane 0, lane 1)
-  auto scatter_batch = [&](const int (&eidx)[U], const Real (&val)[2][U]) {
-    int nn[U];
-    bool ok[2][U];
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int e = eidx[u];
-      nn[u] = n1_0 + (e & (B1 - 1)) + ((e >> logB1) << a.logN1);
-#pragma unroll
-      for (int l = 0; l < 2; ++l) ok[l][u] = e < total && in_range(nn[u], L[l].out_lo, L[l].out_hi);
-    }
-    if (OUT == OUT_TOD) {
-#pragma unroll
-      for (int u = 0; u < U; ++u)
-#pragma unroll
-        for (int l = 0; l < 2; ++l)
-          if (ok[l][u]) static_cast<typename OutT<Real>::type*>(L[l].out)[nn[u]] = to_out(val[l][u]);
-    } else if constexpr (std::is_same<Real, df64>::value && polarised(NS)) {
-      // double-float: round the value to float64 once and weight it with the
-      // float64 (cos, sin) pair (5 float64 operations per sample, not 9)
-      int pp[2][U], qq[2][U], ee[2][U];
-      double2 cs[2][U];
-#pragma unroll
-      for (int u = 0; u < U; ++u)
-#pragma unroll
-        for (int l = 0; l < 2; ++l) {
-          if constexpr (on_the_fly(NS)) {
-            df64 c, sn;
-            load_pointing<Real, NS>(a, L[l], nn[u], ok[l][u], pp[l][u], c, sn);
-            cs[l][u] = make_double2(to_double(c), to_double(sn));
-          } else {
-            pp[l][u] = ok[l][u] ? __ldg(L[l].pix + nn[u]) : -1;
-            cs[l][u] = ok[l][u] ? L[l].cs[nn[u]] : make_double2(0.0, 0.0);
-          }
-          if constexpr (NS == NS_MR) qq[l][u] = ok[l][u] ? __ldg(L[l].pq + nn[u]) : -1;
-          else qq[l][u] = pp[l][u];
-          if constexpr (extended(NS)) ee[l][u] = (ok[l][u] && L[l].pe) ? __ldg(L[l].pe + nn[u]) : -1;
-        }
-#pragma unroll
-      for (int u = 0; u < U; ++u)
-#pragma unroll
-        for (int l = 0; l < 2; ++l) {
-          if (pp[l][u] < 0) continue;
-          double* y = static_cast<double*>(L[l].out);
-          const double v = to_double(val[l][u]);
-          atomicAdd(y + 4LL * pp[l][u], v);
-          atomicAdd(y + 4LL * qq[l][u] + 1, v * cs[l][u].x);
-          atomicAdd(y + 4LL * qq[l][u] + 2, v * cs[l][u].y);
-          if constexpr (extended(NS)) {
-            if (ee[l][u] >= 0) atomic_add_warp(y, 4LL * ee[l][u], v);
-          }
-        }
-    } else {
-      int pp[2][U], qq[2][U];
-      Real cc[2][U], ss[2][U];
-#pragma unroll
-      for (int u = 0; u < U; ++u)
-#pragma unroll
-        for (int l = 0; l < 2; ++l) {
-          load_pointing<Real, NS>(a, L[l], nn[u], ok[l][u], pp[l][u], cc[l][u], ss[l][u]);
-          if constexpr (NS == NS_MR || extended(NS)) {
-            const int* qp = NS == NS_MR ? L[l].pq : L[l].pe;
-            qq[l][u] = (ok[l][u] && qp) ? __ldg(qp + nn[u]) : -1;
-          }
-        }
-      // float32: one atomic per run of samples in one pixel (in float64 and
-      // double-float the shuffles of the partial sums cost more than the
-      // atomics they save)
-      if constexpr (RUNB > 0 && (NS == 1 || NS == 3) && std::is_same<Real, float>::value) {
-        if (a.runs) {
-#pragma unroll
-          for (int u = 0; u < U; ++u)
-#pragma unroll
-            for (int l = 0; l < 2; ++l) {
-              int start;
-              bool tail;
-              run_geometry<RUNB>(pp[l][u], start, tail);
-              const float v = pp[l][u] >= 0 ? val[l][u] : 0.0f;
-              const float s0 = run_sum<RUNB>(v, start);
-              if constexpr (NS == 1) {
-                if (tail && pp[l][u] >= 0) atomicAdd(static_cast<float*>(L[l].out) + pp[l][u], s0);
-              } else {
-                float c = cc[l][u], sn = ss[l][u];
-                finish_angle<float>(c, sn);
-                const float s1 = run_sum<RUNB>(v * c, start), s2 = run_sum<RUNB>(v * sn, start);
-                if (tail && pp[l][u] >= 0)
-                  atomicAdd(reinterpret_cast<float4*>(L[l].out) + pp[l][u], make_float4(s0, s1, s2, 0.0f));
-              }
-            }
-          return;
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < U; ++u)
-#pragma unroll
-        for (int l = 0; l < 2; ++l) {
-          if (pp[l][u] < 0) continue;
-          if constexpr (extended(NS)) {   // the extra column's share (slot 0 of its row)
-            typedef typename OutT<Real>::type Out;
-            if (qq[l][u] >= 0)
-              atomic_add_warp(static_cast<Out*>(L[l].out), (long long)qq[l][u] * (map_ns(NS) == 3 ? 4 : 1),
-                              (Out)to_out(val[l][u]));
-          }
-          Real c = cc[l][u], sn = ss[l][u];
-          if (polarised(NS) && !on_the_fly(NS)) finish_angle<Real>(c, sn);
-          if constexpr (NS == NS_MR)
-            scatter_mr<Real>(static_cast<typename OutT<Real>::type*>(L[l].out), pp[l][u], qq[l][u], val[l][u], c, sn);
-          else
-            scatter<Real, map_ns(NS)>(static_cast<typename OutT<Real>::type*>(L[l].out), pp[l][u], val[l][u], c, sn);
-        }
-    }
-    if constexpr (extended(NS) && OUT == OUT_MAP) {
-      if (a.hwp_base) {   // half-wave-plate parameters, one converged warp at a time
-#pragma unroll
-        for (int u = 0; u < U; ++u)
-#pragma unroll
-          for (int l = 0; l < 2; ++l)
-            hwp_scatter_warp<Real>(hacc + 32 * l, hgrp + l, L[l].pix, L[l].hb, L[l].hang, L[l].htau, nn[u],
-                                   ok[l][u], val[l][u]);
-      }
-    }
-  };
+  auto position = [&](int e) { return e < total ? n1_0 + (e & (B1 - 1)) + ((e >> logB1) << a.logN1) : -1; };
   // float32 with compile-time geometry: the last inverse column pass runs in
   // registers on each thread's two radix-8 groups (see k_f1) before their outputs
   constexpr bool REG3 = sizeof(C) == 8 && LG2 >= 4 && MM_REG_PASS && ELOG == 12 && OP_THREADS == 256 &&
@@ -1096,32 +1106,32 @@ __global__ void __launch_bounds__(256, sizeof(Real) == 4 ? MM_MINB_F13 : MM_MINB
       reg_pass8<C, true>(gv, tw, LG2, base);
 #pragma unroll
       for (int b = 0; b < 8 / U; ++b) {
-        int ee[U];
+        int nn[U];
         Real val[2][U];
 #pragma unroll
         for (int k = 0; k < U; ++k) {
-          ee[k] = threadIdx.x + (2 * (U * b + k) + G) * bd;
+          nn[k] = position(threadIdx.x + (2 * (U * b + k) + G) * bd);
           val[0][k] = gv[U * b + k].x;
           val[1][k] = gv[U * b + k].y;
         }
-        scatter_batch(ee, val);
+        scatter_samples<Real, NS, OUT, U, RUNB>(a, L, nn, val, hacc, hgrp);
       }
     }
   } else {
     for (int e0 = threadIdx.x; e0 < total; e0 += bd * U) {
-      int ee[U];
+      int nn[U];
       Real val[2][U];
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         const int e = e0 + u * bd;
-        ee[u] = e;
+        nn[u] = position(e);
         C z;
         z.x = z.y = 0;
         if (e < total) z = buf[(e & (B1 - 1)) * rs + swz<SW>(e >> logB1)];
         val[0][u] = z.x;
         val[1][u] = z.y;
       }
-      scatter_batch(ee, val);
+      scatter_samples<Real, NS, OUT, U, RUNB>(a, L, nn, val, hacc, hgrp);
     }
   }
   if constexpr (HWP) {
@@ -1134,6 +1144,8 @@ __global__ void __launch_bounds__(256, sizeof(Real) == 4 ? MM_MINB_F13 : MM_MINB
   }
 }
 
+
+#include "operator_reg.cuh"  // k_c1, k_c2, k_c3 (float32)
 
 // ---------------------------------------------------------------- k_diag
 // White noise (one filter lag, e.g. destriping runs, Section 6 item 3): N^-1
@@ -1322,6 +1334,16 @@ OpKernels pick_kernels(const Plan* p) {
   if constexpr (generic_only) {
     k.f1 = k_f1<Real, NS, IN, 0>;
     k.f3 = k_f3<Real, NS, OUT, 0>;
+  } else if constexpr (std::is_same<Real, float>::value) {
+    // lengths 2^14 .. 2^18 run in operator_reg.cuh: the others' columns have
+    // 128 (2^13), 512 (2^19 with fft_split) or 1024 points, or few enough for
+    // the generic instance
+    switch (p->logN2) {
+      case 7: k.f1 = k_f1<Real, NS, IN, 7>; k.f3 = k_f3<Real, NS, OUT, 7>; break;
+      case 9: k.f1 = k_f1<Real, NS, IN, 9>; k.f3 = k_f3<Real, NS, OUT, 9>; break;
+      case 10: k.f1 = k_f1<Real, NS, IN, 10>; k.f3 = k_f3<Real, NS, OUT, 10>; break;
+      default: k.f1 = k_f1<Real, NS, IN, 0>; k.f3 = k_f3<Real, NS, OUT, 0>; break;
+    }
   } else {
     switch (p->logN2) {
       case 7: k.f1 = k_f1<Real, NS, IN, 7>; k.f3 = k_f3<Real, NS, OUT, 7>; break;
@@ -1331,13 +1353,22 @@ OpKernels pick_kernels(const Plan* p) {
       default: k.f1 = k_f1<Real, NS, IN, 0>; k.f3 = k_f3<Real, NS, OUT, 0>; break;
     }
   }
-  switch (p->logN1) {
-    case 6: k.f2 = k_f2<Real, 6>; break;
-    case 7: k.f2 = k_f2<Real, 7>; break;
-    case 8: k.f2 = k_f2<Real, 8>; break;
-    case 9: k.f2 = k_f2<Real, 9>; break;
-    case 10: k.f2 = k_f2<Real, 10>; break;
-    default: k.f2 = k_f2<Real, 0>; break;
+  if constexpr (std::is_same<Real, float>::value) {
+    switch (p->logN1) {
+      case 6: k.f2 = k_f2<Real, 6>; break;
+      case 9: k.f2 = k_f2<Real, 9>; break;
+      case 10: k.f2 = k_f2<Real, 10>; break;
+      default: k.f2 = k_f2<Real, 0>; break;
+    }
+  } else {
+    switch (p->logN1) {
+      case 6: k.f2 = k_f2<Real, 6>; break;
+      case 7: k.f2 = k_f2<Real, 7>; break;
+      case 8: k.f2 = k_f2<Real, 8>; break;
+      case 9: k.f2 = k_f2<Real, 9>; break;
+      case 10: k.f2 = k_f2<Real, 10>; break;
+      default: k.f2 = k_f2<Real, 0>; break;
+    }
   }
   return k;
 }
@@ -1496,12 +1527,21 @@ madmap_status launch_all(Plan* p, const void* in, void* out, long long in_stride
   a.runs = p->runs;
   a.tiles = ts ? ts->tiles : p->tiles;
   const int n_tiles = ts ? ts->n_tiles : p->n_tiles;
+  constexpr bool F32 = std::is_same<Real, float>::value;
+  const bool reg = F32 && p->reg.logN1 > 0;   // register transforms (static shared memory)
   const size_t sm13 = smem_f13<Real>(p), sm2 = smem_f2<Real>(p);
   const OpKernels K = pick_kernels<Real, NS, IN, OUT>(p);
+  a.reg_logN1 = p->reg.logN1;
+  a.reg_col = p->reg.col;
+  a.reg_row = p->reg.row;
+  a.reg_four = p->reg.four;
+  a.reg_four0 = p->reg.four0;
   // n_rhs == 0 only sets the kernels' attributes, so it can precede a capture
-  MM_CUDA(set_smem(K.f1, sm13));
-  MM_CUDA(set_smem(K.f3, sm13));
-  MM_CUDA(set_smem(K.f2, sm2));
+  if (!reg) {
+    MM_CUDA(set_smem(K.f1, sm13));
+    MM_CUDA(set_smem(K.f3, sm13));
+    MM_CUDA(set_smem(K.f2, sm2));
+  }
   if (p->diag && !ts) {
     // white noise: one diagonal pass per right-hand side (launch events as
     // four per application so per-kernel timing keeps its layout)
@@ -1566,6 +1606,12 @@ madmap_status launch_all(Plan* p, const void* in, void* out, long long in_stride
         const cudaStream_t cs = pipe ? p->op_stream[chunk & 1] : s;
         a.scratch = static_cast<char*>(p->scratch) + (pipe ? (size_t)(chunk & 1) * slot_bytes : 0);
         ++chunk;
+        if constexpr (F32) {
+          if (reg) {
+            launch_reg<NS, IN, OUT>(a, nt, cs, ev, &ei);
+            continue;
+          }
+        }
         dim3 g13(p->N1 / a.B1, nt), g2(p->N2 / a.B2, nt);
         if (ev) cudaEventRecord(ev[ei++], s);
         K.f1<<<g13, OP_THREADS, sm13, cs>>>(a);
@@ -1738,33 +1784,6 @@ madmap_status impl_time(Plan* p, const void* in, void* out, int reps, double ms[
 #undef MM_TIME
 }
 
-// Resident CTAs per SM of the map-to-map kernels (the least of the three) and
-// CTAs per tile of the column kernels, for wave-aligned chunk sizes.
-template <typename Real>
-void impl_occupancy(const Plan* p, int& ctas_per_sm, int& ctas_per_tile) {
-  int b1 = 0, b2 = 0, n1 = 0, n2 = 0, n3 = 0;
-  geometry<Real>(p, b1, b2);
-  const size_t s13 = smem_f13<Real>(p), s2 = smem_f2<Real>(p);
-  const int k = layout(p);
-#define MM_PICK(NSV) pick_kernels<Real, NSV, IN_MAPX, OUT_MAP>(p)
-  const OpKernels K = MM_FOR_LAYOUT(k, MM_PICK);
-#undef MM_PICK
-  set_smem(K.f1, s13);
-  set_smem(K.f2, s2);
-  set_smem(K.f3, s13);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n1, K.f1, OP_THREADS, s13);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n2, K.f2, OP_THREADS, s2);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n3, K.f3, OP_THREADS, s13);
-  cudaGetLastError();
-  ctas_per_sm = std::max(1, std::min(n1, std::min(n2, n3)));
-  ctas_per_tile = std::max(1, p->N1 / std::max(1, b1));
-}
-
-template <typename Real>
-size_t impl_f13_smem(const Plan* p) {
-  return smem_f13<Real>(p);
-}
-
 template <typename Real>
 madmap_status impl_weights(long long n, const float* psi, void* c, void* s, cudaStream_t st) {
   if constexpr (std::is_same<Real, df64>::value) {
@@ -1787,9 +1806,6 @@ OpImpl make_impl() {
   t.launch = impl_launch<Real>;
   t.launch_set = impl_launch_set<Real>;
   t.time = impl_time<Real>;
-  if constexpr (std::is_same<Real, df64>::value) t.occupancy = nullptr;
-  else t.occupancy = impl_occupancy<Real>;
-  t.f13_smem = impl_f13_smem<Real>;
   return t;
 }
 

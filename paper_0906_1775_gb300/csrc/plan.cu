@@ -82,6 +82,7 @@ static void free_windows(Plan* p) {
   p->Hdf = nullptr;
   p->tw64 = nullptr;
   p->tw32 = nullptr;
+  p->reg = RegTables();
   p->twdf = nullptr;
   p->scratch = nullptr;
 }
@@ -976,6 +977,46 @@ static int choose_fft_len(const std::vector<long long>& off, const std::vector<i
   return bestM;
 }
 
+// ---------------------------------------------------------------- register transforms
+size_t reg_table_floats(int logN1) { return 16 * 8 + 32 * 16 + (size_t)(1 << logN1) * (8 + 32); }
+
+void reg_fill_tables(int logN1, float* o) {
+  const long long N1 = 1LL << logN1, M = REG_N2 * N1;
+  auto put = [&](long long num, long long den) {   // exp(-2 pi i num / den)
+    const double ang = 2.0 * M_PI * (double)(num % den) / (double)den;
+    *o++ = (float)cos(ang);
+    *o++ = (float)-sin(ang);
+  };
+  for (int j = 0; j < 16; ++j)
+    for (int k = 0; k < 4; ++k) put(j << k, REG_N2);
+  for (int l = 0; l < 32; ++l) {
+    for (int k = 0; k < 5; ++k) put(l << k, N1);
+    for (int k = 0; k < 6; ++k) *o++ = 0.f;
+  }
+  for (long long n = 0; n < N1; ++n)
+    for (int k = 0; k < 4; ++k) put((16 * n) << k, M);
+  for (long long p = 0; p < 16; ++p)
+    for (long long n = 0; n < N1; ++n) put(n * p, M);
+}
+
+RegTables reg_point_tables(int logN1, const float* base) {
+  RegTables t;
+  t.logN1 = logN1;
+  t.col = reinterpret_cast<const float4*>(base);
+  t.row = t.col + 16 * 2;
+  t.four = t.row + 32 * 4;
+  t.four0 = reinterpret_cast<const float2*>(t.four + 2 * (1 << logN1));
+  return t;
+}
+
+// The spectrum re (length 256 N1) as the register kernels read it: [k2][k1], / M.
+void reg_spectrum(const std::vector<double>& re, int logN1, float* h32) {
+  const int N1 = 1 << logN1;
+  const double M = (double)REG_N2 * N1;
+  for (int k2 = 0; k2 < REG_N2; ++k2)
+    for (int k1 = 0; k1 < N1; ++k1) h32[(size_t)k2 * N1 + k1] = (float)(re[k2 + (size_t)REG_N2 * k1] / M);
+}
+
 // Spectrum of one filter's circulant embedding into h64/h32/hdf (the layout
 // the row kernel reads); returns false when the symbol is not positive.
 static bool filter_spectrum(const Plan* p, int f, double* h64, float* h32, df64* hdf, double* min_out) {
@@ -1005,6 +1046,7 @@ static bool filter_spectrum(const Plan* p, int f, double* h64, float* h32, df64*
       hdf[o] = df64(v);
     }
   }
+  if (p->reg.logN1 > 0) reg_spectrum(re, p->reg.logN1, h32);
   return true;
 }
 
@@ -1299,6 +1341,15 @@ static madmap_status setup_windows(Plan* p, int M, long long tpc_req, cudaStream
   if ((st = walloc_t(p, &p->H64, (size_t)p->n_filters * p->M)) != MADMAP_OK) return st;
   if ((st = walloc_t(p, &p->H32, (size_t)p->n_filters * p->M)) != MADMAP_OK) return st;
   if ((st = walloc_t(p, &p->Hdf, (size_t)p->n_filters * p->M)) != MADMAP_OK) return st;
+  const int rl = reg_log_n1(p->M);
+  if (rl > 0) {
+    float* tab = nullptr;
+    std::vector<float> h(reg_table_floats(rl));
+    reg_fill_tables(rl, h.data());
+    if ((st = walloc_t(p, &tab, h.size())) != MADMAP_OK) return st;
+    MM_CUDA(cudaMemcpy(tab, h.data(), sizeof(float) * h.size(), cudaMemcpyHostToDevice));
+    p->reg = reg_point_tables(rl, tab);
+  }
   if ((st = build_spectra(p)) != MADMAP_OK) return st;
   {
     std::vector<double2> t64(p->M);
@@ -1312,10 +1363,10 @@ static madmap_status setup_windows(Plan* p, int M, long long tpc_req, cudaStream
       tdf[j].y = df64(t64[j].y);
     }
     if ((st = walloc_t(p, &p->tw64, p->M)) != MADMAP_OK) return st;
-    if ((st = walloc_t(p, &p->tw32, p->M)) != MADMAP_OK) return st;
+    if (rl == 0 && (st = walloc_t(p, &p->tw32, p->M)) != MADMAP_OK) return st;
     if ((st = walloc_t(p, &p->twdf, p->M)) != MADMAP_OK) return st;
     MM_CUDA(cudaMemcpy(p->tw64, t64.data(), sizeof(double2) * p->M, cudaMemcpyHostToDevice));
-    MM_CUDA(cudaMemcpy(p->tw32, t32.data(), sizeof(float2) * p->M, cudaMemcpyHostToDevice));
+    if (rl == 0) MM_CUDA(cudaMemcpy(p->tw32, t32.data(), sizeof(float2) * p->M, cudaMemcpyHostToDevice));
     MM_CUDA(cudaMemcpy(p->twdf, tdf.data(), sizeof(cdf64) * p->M, cudaMemcpyHostToDevice));
   }
   {

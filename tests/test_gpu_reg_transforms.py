@@ -1,0 +1,57 @@
+"""The float32 register transforms (window lengths 2^14 to 2^18).
+
+Every row length N1 = M / 256 of 64 to 1024 points runs its own kernel; the
+lengths just outside (2^13, 2^19) run the shared-memory ones.  Each length's
+N^-1 is checked against the Eq. 15 direct sum on intervals that end inside,
+at and past a window's exact part, and its operator (gather and scatter of both
+paired windows, an odd number of them, flagged samples) against the oracle.
+
+Tolerance: a float32 transform of 2^18 points and its inverse pass 36 radix-2
+levels; each level and each twiddle product adds at most about two roundings
+of 2^-24, and they add up as a random walk: 2^-24 * 2 * sqrt(2 * 36) = 1e-6.
+"""
+
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+from tests.gpu_helpers import cuda, host, make_plan
+from tests.helpers import lags_for, rel_rms, system_for, tiny_IQU, tiny_T
+
+pytestmark = pytest.mark.gpu
+
+TOL = 1e-6
+
+
+@pytest.mark.parametrize("lg", range(13, 20))
+def test_weighting_matches_direct_sum(lg):
+    import torch
+    from oracle.noise import apply_ninv_direct
+    M, n_lags = 1 << lg, 129
+    exact = M - 2 * (n_lags - 1)     # samples one window weighs exactly
+    p = tiny_T(seed=90 + lg, n=4 * exact + 777, width=24, n_lags=n_lags, ivls=(1, 775, exact, exact + 1, 2 * exact))
+    plan = make_plan(p, fft_len=M)
+    assert plan.stats["fft_len"] == M
+    y = np.random.default_rng(lg).standard_normal(p.n_samples).astype(np.float32)
+    ref = apply_ninv_direct(y.astype(np.float64), p.interval_offsets, p.interval_filter, lags_for(p))
+    w = host(plan.apply_ninv(cuda(y, torch.float32), precision="fp32"))[0]
+    assert rel_rms(w, ref) < TOL, rel_rms(w, ref)
+    for i in range(len(p.interval_filter)):
+        a, b = int(p.interval_offsets[i]), int(p.interval_offsets[i + 1])
+        assert rel_rms(w[a:b], ref[a:b]) < 4 * TOL, i    # single samples carry no averaging
+
+
+@pytest.mark.parametrize("lg", range(14, 19))
+@pytest.mark.parametrize("runs", [-1, 1])
+def test_operator_matches_oracle(lg, runs):
+    import torch
+    p = tiny_IQU(seed=95, n_per_det=7001, n_lags=300, n_ivl_lo=200, n_ivl_hi=5000, flag_frac=0.02)
+    S = system_for(p)
+    plan = make_plan(p, fft_len=1 << lg, scatter_runs=runs)
+    x = np.random.default_rng(lg).standard_normal((S.n_obs, 3)).astype(np.float32)
+    x[S.excised] = 0.0
+    y = host(plan.apply_ATNA(cuda(x, torch.float32), precision="fp32"))[0]
+    assert rel_rms(y, S.H(x.astype(np.float64))) < 2 * TOL   # two weights and a sum more per sample
+    b = host(plan.rhs(cuda(p.d), precision="fp32"))[0]
+    assert rel_rms(b, S.rhs(p.d[0])) < 2 * TOL
