@@ -20,9 +20,12 @@
 // on half of 97 tiles of 2^17 (IQU, 512 x 512 raster): columns 67.7 -> 50.2 and
 // 61.5 -> 59.1 us, rows 30.9 -> 23.6 us, one application 262 -> 213 us; on 103
 // tiles of 2^18 (ring scan, N_side 512): 109 -> 77, 121 -> 112 and 65 -> 47 us,
-// 531 -> 412 us.  Sixteen columns a CTA because 256 threads x 16 elements leave
+// 531 -> 412 us (and to 201 and 365 us with the packed sums and short run sums
+below).  Sixteen columns a CTA because 256 threads x 16 elements leave
 // four CTAs per SM at 64 registers; three CTAs with twice or four times the
-// loads in flight per thread measured slower (442 and 468 us on the ring scan).
+// loads in flight per thread measured slower (442 and 468 us on the ring scan),
+and so did loading the pointing one to four batches ahead of the map (373 -> 387
+to 458 us: at 64 registers the loads in flight cost more than they hide).
 // Shorter windows would leave rows of less than 64 points to groups of fewer
 // than 8 lanes (32-byte rows of scratch), longer ones need rows of more than
 // 32 x 32: both stay with k_f1, k_f2 and k_f3.
@@ -52,6 +55,19 @@ __device__ __forceinline__ float2 mul_w32(float2 v, int k) {
   return make_float2(v.x * c + v.y * s, v.y * c - v.x * s);
 }
 
+// Complex sums, one packed instruction each (two float32 lanes of the register
+// pair, rounded as the scalar sums): the row kernel issues on 69% of its cycles
+// and half of its instructions were these (ring scan, 2^18: rows 46.7 -> 42.5,
+// inverse columns 113 -> 103 us per launch, one application 416 -> 387 us).
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) {
+  unsigned long long r;
+  asm("sub.rn.f32x2 %0, %1, %2;"
+      : "=l"(r)
+      : "l"(reinterpret_cast<const unsigned long long&>(a)), "l"(reinterpret_cast<const unsigned long long&>(b)));
+  return reinterpret_cast<const float2&>(r);
+}
+
 // 2^LG-point DFT (INV: inverse, unnormalised) of registers, natural order in,
 // bit-reversed order out: radix-2 decimation in frequency, constant twiddles.
 template <int LG, bool INV>
@@ -63,8 +79,8 @@ __device__ __forceinline__ void reg_dft(float2 (&v)[1 << LG]) {
     for (int m = 0; m < (1 << LG); ++m) {
       if ((m & span) == 0) {
         const float2 x = v[m], y = v[m + span];
-        v[m] = cadd(x, y);
-        v[m + span] = mul_w32<INV>(csub(x, y), ((m & (span - 1)) << st) << (5 - LG));
+        v[m] = add2(x, y);
+        v[m + span] = mul_w32<INV>(sub2(x, y), ((m & (span - 1)) << st) << (5 - LG));
       }
     }
   }
@@ -108,6 +124,13 @@ struct Powers {
   }
 };
 
+// Lanes of a run sum in k_c3 (run_sum): a run of samples in one pixel adds once
+// per aligned group of this many.  Four takes two shuffle steps of each of the
+// three sums where a warp row of 16 samples takes four, for one atomic in two
+// samples instead of one in three on the ring scan (0.65 repeats); the shuffles
+// were a third of the kernel's L1 wavefronts (16, 8, 4 lanes: 103.5, 97.9, 97.6
+// us per launch, 387, 377, 373 us per application).
+constexpr int REG_RUN = 4;
 constexpr int REG_COLS = 16;   // columns per CTA of k_c1 and k_c3 (256 threads x 16 elements)
 #ifndef MM_MINB_C1
 #define MM_MINB_C1 4
@@ -297,7 +320,7 @@ __global__ void __launch_bounds__(256, MM_MINB_C3) k_c3(OpArgs a) {
       val[0][k] = y[U * b + k].x;
       val[1][k] = y[U * b + k].y;
     }
-    scatter_samples<float, NS, OUT, U, REG_COLS>(a, L, nn, val, hacc, hgrp);
+    scatter_samples<float, NS, OUT, U, REG_RUN>(a, L, nn, val, hacc, hgrp);
   }
   if constexpr (HWP) {
     if (a.hwp_base) {
