@@ -24,8 +24,8 @@
 // below).  Sixteen columns a CTA because 256 threads x 16 elements leave
 // four CTAs per SM at 64 registers; three CTAs with twice or four times the
 // loads in flight per thread measured slower (442 and 468 us on the ring scan),
-and so did loading the pointing one to four batches ahead of the map (373 -> 387
-to 458 us: at 64 registers the loads in flight cost more than they hide).
+// and so did loading the pointing one to four batches ahead of the map (373 -> 387
+// to 458 us: at 64 registers the loads in flight cost more than they hide).
 // Shorter windows would leave rows of less than 64 points to groups of fewer
 // than 8 lanes (32-byte rows of scratch), longer ones need rows of more than
 // 32 x 32: both stay with k_f1, k_f2 and k_f3.
