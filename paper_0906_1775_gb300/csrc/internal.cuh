@@ -54,6 +54,13 @@ struct DiagItem {
   int filter, pad;
 };
 
+// Scratch of one launch of a tile set: four waves of the float32 column
+// kernels' CTAs (152 SMs x 4 CTAs x 4096 elements) at 16 bytes an element.  A
+// set's own chunks instead of the plan's, which are sized for one right-hand
+// side (16 right-hand sides of 2.5e6 samples, M = 2^16: 31 launches of 208 CTAs
+// for 608 resident ones).
+constexpr size_t BATCH_SLOT_BYTES = (size_t)4 * 152 * 4 * 4096 * 16;
+
 // A list of tiles whose lanes name their right-hand side (batched solves).
 struct TileSet {
   Tile* tiles = nullptr;  // device
@@ -355,6 +362,11 @@ struct Plan {
   // An application of several chunks alternates them between two streams,
   // each with its own scratch slot, so one chunk's kernels overlap the
   // previous chunk's tail and its scratch and pointing stay in L2.
+  bool tpc_fixed = false;          // tiles_per_chunk set by the description
+  // Tile sets (batched solves) run in chunks of their own, two slots of
+  // BATCH_SLOT_BYTES allocated once by the first set larger than a plan chunk.
+  void* batch_scratch = nullptr;
+  bool batch_tried = false;
   cudaStream_t op_stream[2] = {nullptr, nullptr};
   cudaEvent_t op_fork = nullptr;
   cudaEvent_t op_join[2] = {nullptr, nullptr};
@@ -450,8 +462,9 @@ madmap_status op_launch(Plan* p, int prec, int in_mode, int out_mode, const void
 // duration of one application as the solver launches it.
 madmap_status op_time(Plan* p, int prec, const void* in, void* out, int reps, double ms[4], cudaStream_t s);
 
-// Number of operator launches per application and tiles per launch.
-void chunking(const Plan* p, int& n_chunks, int& per_chunk, int n_tiles = -1);
+// Number of operator launches per application and tiles per launch; n_tiles of
+// a tile set with `cap` tiles a launch, or (the default) the plan's own.
+void chunking(const Plan* p, int& n_chunks, int& per_chunk, int n_tiles = -1, int cap = 0);
 
 // The operator over a tile set (lanes carry their rhs; per-rhs strides in
 // elements; skip[rhs * skip_stride], if skip is not NULL, marks right-hand

@@ -1567,18 +1567,29 @@ madmap_status launch_all(Plan* p, const void* in, void* out, long long in_stride
     MM_CUDA(cudaGetLastError());
     return MADMAP_OK;
   }
+  // scratch slots of this launch: the plan's, or a tile set's own (at least
+  // two chunks from 16 tiles on, so that the two streams overlap)
+  char* scratch = static_cast<char*>(p->scratch);
+  size_t slot_bytes = (size_t)p->tiles_per_chunk * p->M * sizeof(double2);
+  int slots = p->scratch_slots, cap = 0;
+  if (ts && p->batch_scratch) {
+    scratch = static_cast<char*>(p->batch_scratch);
+    slot_bytes = BATCH_SLOT_BYTES;
+    slots = 2;
+    cap = (int)std::min<size_t>(slot_bytes / ((size_t)p->M * sizeof(typename CxT<Real>::type)), 65535);
+    if (n_tiles >= 16) cap = std::min(cap, (n_tiles + 1) / 2);
+  }
   int n_chunks, per_chunk;
-  chunking(p, n_chunks, per_chunk, n_tiles);
+  chunking(p, n_chunks, per_chunk, n_tiles, cap);
   // map replicas for small, heavily hit maps (single right-hand side per launch)
   typedef typename OutT<Real>::type Out;
   const bool use_rep = !ts && OUT == OUT_MAP && p->n_rep > 1 && p->rep;
   const long long n_map = (long long)std::max(1, p->n_obs) * p->ns_pad;
   // several chunks: alternate two streams (own scratch slot each) so chunks overlap
   // (with replicas only when one application is enqueued: the replicas are reused)
-  const bool pipe = !ev && n_rhs > 0 && n_chunks > 1 && p->op_stream[0] && p->scratch_slots > 1 &&
+  const bool pipe = !ev && n_rhs > 0 && n_chunks > 1 && p->op_stream[0] && slots > 1 &&
                     (!use_rep || n_rhs * reps == 1);
   const int rgrid = (int)std::min<long long>((n_map + 255) / 256, 152LL * 8);
-  const size_t slot_bytes = (size_t)p->tiles_per_chunk * p->M * sizeof(double2);
   if (pipe) {
     MM_CUDA(cudaEventRecord(p->op_fork, s));
     for (int i = 0; i < 2; ++i) MM_CUDA(cudaStreamWaitEvent(p->op_stream[i], p->op_fork, 0));
@@ -1604,7 +1615,7 @@ madmap_status launch_all(Plan* p, const void* in, void* out, long long in_stride
         const int nt = (n_tiles - t0) < per_chunk ? (n_tiles - t0) : per_chunk;
         a.tile0 = t0;
         const cudaStream_t cs = pipe ? p->op_stream[chunk & 1] : s;
-        a.scratch = static_cast<char*>(p->scratch) + (pipe ? (size_t)(chunk & 1) * slot_bytes : 0);
+        a.scratch = scratch + (pipe ? (size_t)(chunk & 1) * slot_bytes : 0);
         ++chunk;
         if constexpr (F32) {
           if (reg) {

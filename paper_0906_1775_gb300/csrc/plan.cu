@@ -896,6 +896,17 @@ static madmap_status build_det_rows(Plan* p, cudaStream_t s) {
   return ensure_wtod(p, 1);
 }
 
+// The two streams (and their events) that chunks alternate between.
+static madmap_status ensure_op_streams(Plan* p) {
+  if (p->op_stream[0]) return MADMAP_OK;
+  for (int i = 0; i < 2; ++i) {
+    MM_CUDA(cudaStreamCreateWithFlags(&p->op_stream[i], cudaStreamNonBlocking));
+    MM_CUDA(cudaEventCreateWithFlags(&p->op_join[i], cudaEventDisableTiming));
+  }
+  MM_CUDA(cudaEventCreateWithFlags(&p->op_fork, cudaEventDisableTiming));
+  return MADMAP_OK;
+}
+
 madmap_status get_tile_set(Plan* p, int n_rhs, TileSet** out) {
   if (p->det) {
     madmap_status st = ensure_wtod(p, n_rhs);
@@ -949,6 +960,13 @@ madmap_status get_tile_set(Plan* p, int n_rhs, TileSet** out) {
       delete t;
       return cuda_fail(e, "cudaMemcpy (tile set)");
     }
+  }
+  if (!p->batch_tried && !p->tpc_fixed && t->n_tiles > p->tiles_per_chunk &&
+      (size_t)p->tiles_per_chunk * p->M * sizeof(double2) < BATCH_SLOT_BYTES) {
+    // larger chunks for tile sets; without the memory they run in the plan's
+    p->batch_tried = true;
+    if (ensure_op_streams(p) == MADMAP_OK && dalloc(p, &p->batch_scratch, 2 * BATCH_SLOT_BYTES) != MADMAP_OK)
+      p->batch_scratch = nullptr;
   }
   p->tile_sets.push_back(t);
   *out = t;
@@ -1372,13 +1390,7 @@ static madmap_status setup_windows(Plan* p, int M, long long tpc_req, cudaStream
   {
     const int n_chunks = p->n_tiles ? (p->n_tiles + p->tiles_per_chunk - 1) / p->tiles_per_chunk : 0;
     p->scratch_slots = n_chunks > 1 ? 2 : 1;
-    if (n_chunks > 1 && !p->op_stream[0]) {
-      for (int i = 0; i < 2; ++i) {
-        MM_CUDA(cudaStreamCreateWithFlags(&p->op_stream[i], cudaStreamNonBlocking));
-        MM_CUDA(cudaEventCreateWithFlags(&p->op_join[i], cudaEventDisableTiming));
-      }
-      MM_CUDA(cudaEventCreateWithFlags(&p->op_fork, cudaEventDisableTiming));
-    }
+    if (n_chunks > 1 && (st = ensure_op_streams(p)) != MADMAP_OK) return st;
   }
   return walloc(p, &p->scratch, (size_t)p->scratch_slots * p->tiles_per_chunk * p->M * sizeof(double2));
 }
@@ -1839,6 +1851,7 @@ extern "C" madmap_status madmap_plan_create(const madmap_plan_desc* d, void* str
     MM_TRYC(cudaStreamSynchronize(s));
     p->repeat_frac = (double)h / (double)p->n_t;
   }
+  p->tpc_fixed = d->tiles_per_chunk > 0;
   p->runs_fixed = d->scatter_runs != 0;
   p->split_down = d->fft_split;
   p->split_fixed = d->fft_split != 0;
