@@ -117,20 +117,36 @@ void host_fft(std::vector<double>& re, std::vector<double>& im, bool inverse) {
       std::swap(im[i], im[j]);
     }
   }
+  if (n < 2) return;
+  // cos and sin of 2 pi k / n for k < n/2, from the first octant by symmetry
   const double sgn = inverse ? 1.0 : -1.0;
-  for (size_t len = 2; len <= n; len <<= 1) {
-    const size_t half = len >> 1;
-    std::vector<double> wr(half), wi(half);
-    for (size_t k = 0; k < half; ++k) {
-      const double ang = 2.0 * M_PI * (double)k / (double)len;
-      wr[k] = cos(ang);
-      wi[k] = sgn * sin(ang);
+  const size_t h = n / 2;
+  std::vector<double> wr(h), wi(h);
+  for (size_t k = 0; k < h; ++k) {
+    const size_t q = n / 4;                      // a quarter turn
+    const bool second = q > 0 && k > q;          // (pi/2, pi): cos(pi - x) = -cos x
+    const size_t r = second ? h - k : k;
+    double c, si;
+    if (8 * r <= n) {
+      const double ang = 2.0 * M_PI * (double)r / (double)n;
+      c = second ? -wr[r] : cos(ang);
+      si = second ? sgn * wi[r] : sin(ang);
+    } else {                                     // cos x = sin(pi/2 - x)
+      c = sgn * wi[q - r];
+      si = wr[q - r];
+      if (second) c = -c;
     }
+    wr[k] = c;
+    wi[k] = sgn * si;
+  }
+  for (size_t len = 2; len <= n; len <<= 1) {
+    const size_t half = len >> 1, st = n / len;
     for (size_t i = 0; i < n; i += len) {
       for (size_t k = 0; k < half; ++k) {
         const size_t a = i + k, b = a + half;
-        const double xr = re[b] * wr[k] - im[b] * wi[k];
-        const double xi = re[b] * wi[k] + im[b] * wr[k];
+        const double c = wr[k * st], d = wi[k * st];
+        const double xr = re[b] * c - im[b] * d;
+        const double xi = re[b] * d + im[b] * c;
         re[b] = re[a] - xr;
         im[b] = im[a] - xi;
         re[a] += xr;
@@ -143,6 +159,13 @@ void host_fft(std::vector<double>& re, std::vector<double>& im, bool inverse) {
 static bool is_pow2(long long v) { return v > 0 && (v & (v - 1)) == 0; }
 
 // ---------------------------------------------------------------- noise filter
+// cos(2 pi j / L), j < L.
+static std::vector<double> cos_table(size_t L) {
+  std::vector<double> c(L);
+  for (size_t j = 0; j < L; ++j) c[j] = cos(2.0 * M_PI * (double)j / (double)L);
+  return c;
+}
+
 // Inverse DFT of an even real sequence q of length L, first n outputs.
 static void even_idft(const std::vector<double>& q, int n, double* out) {
   const size_t L = q.size();
@@ -151,12 +174,63 @@ static void even_idft(const std::vector<double>& q, int n, double* out) {
     host_fft(re, im, true);
     for (int t = 0; t < n; ++t) out[t] = re[t] / (double)L;
   } else {
+    const std::vector<double> ct = cos_table(L);
     for (int t = 0; t < n; ++t) {
       double acc = 0.0;
-      for (size_t j = 0; j < L; ++j) acc += q[j] * cos(2.0 * M_PI * (double)((j * (size_t)t) % L) / (double)L);
+      size_t k = 0;                              // (j t) mod L
+      for (size_t j = 0; j < L; ++j) {
+        acc += q[j] * ct[k];
+        k += (size_t)t;
+        if (k >= L) k -= L;
+      }
       out[t] = acc / (double)L;
     }
   }
+}
+
+// Its transpose: sum_t x_t cos(2 pi j t / L) for j = 0 .. L/2.
+static void even_idft_transpose(const double* x, int n, size_t L, double* out) {
+  if (is_pow2((long long)L)) {
+    std::vector<double> re(L, 0.0), im(L, 0.0);
+    for (int t = 0; t < n; ++t) re[t] = x[t];
+    host_fft(re, im, false);
+    for (size_t j = 0; j <= L / 2; ++j) out[j] = re[j];
+  } else {
+    const std::vector<double> ct = cos_table(L);
+    for (size_t j = 0; j <= L / 2; ++j) {
+      double acc = 0.0;
+      size_t k = 0;
+      for (int t = 0; t < n; ++t) {
+        acc += x[t] * ct[k];
+        k += j;
+        if (k >= L) k -= L;
+      }
+      out[j] = acc;
+    }
+  }
+}
+
+// 1 / PSD at the L = 4 n_lags frequencies, by symmetry from the first half
+// (j <= L/2; the zero frequency takes the first one's value), and (f_knee / nu)^alpha.
+static void inverse_psd(int L, double fs, double sigma, double fknee, double alpha, std::vector<double>& q,
+                        std::vector<double>& r) {
+  q.resize(L / 2 + 1);
+  r.resize(L / 2 + 1);
+  for (int j = 1; j <= L / 2; ++j) {
+    r[j] = pow(fknee / ((double)j * fs / (double)L), alpha);
+    q[j] = 1.0 / (sigma * sigma * (1.0 + r[j]));
+  }
+  r[0] = r[1];
+  q[0] = q[1];
+}
+
+// d(1 / PSD) / d(sigma, f_knee, alpha)[k] at frequency j.
+static double inverse_psd_grad(int k, int j, int L, double fs, double sigma, double fknee, double alpha, double q,
+                               double r) {
+  if (k == 0) return -2.0 * q / sigma;
+  if (!(fknee > 0)) return 0.0;
+  if (k == 1) return -q * q * sigma * sigma * alpha * r / fknee;
+  return -q * q * sigma * sigma * r * log(fknee / ((double)std::max(1, j) * fs / (double)L));
 }
 
 }  // namespace mm
@@ -169,39 +243,38 @@ extern "C" madmap_status madmap_noise_filter(int32_t n_lags, double fs, double s
   MM_CHECK(fs > 0 && sigma > 0 && fknee >= 0 && isfinite(alpha), MADMAP_ERR_INVALID_ARG,
            "noise_filter: need fs > 0, sigma > 0, fknee >= 0, finite alpha");
   const int L = 4 * n_lags;
-  std::vector<double> nu(L), q(L);
-  for (int j = 0; j < L; ++j) nu[j] = (double)std::min(j, L - j) * fs / (double)L;
-  nu[0] = nu[1];
-  for (int j = 0; j < L; ++j) q[j] = 1.0 / (sigma * sigma * (1.0 + pow(fknee / nu[j], alpha)));
-  std::vector<double> c(n_lags);
-  even_idft(q, n_lags, c.data());
-  for (int t = 0; t < n_lags; ++t) lags_out[t] = (1.0 - (double)t / n_lags) * c[t];
-  if (dlags_out) {
-    std::vector<double> dq(L);
-    for (int k = 0; k < 3; ++k) {
-      for (int j = 0; j < L; ++j) {
-        const double r = pow(fknee / nu[j], alpha);
-        if (k == 0) dq[j] = -2.0 * q[j] / sigma;
-        else if (k == 1) dq[j] = fknee > 0 ? -q[j] * q[j] * sigma * sigma * alpha * r / fknee : 0.0;
-        else dq[j] = fknee > 0 ? -q[j] * q[j] * sigma * sigma * r * log(fknee / nu[j]) : 0.0;
-      }
-      even_idft(dq, n_lags, c.data());
-      for (int t = 0; t < n_lags; ++t) dlags_out[k * n_lags + t] = (1.0 - (double)t / n_lags) * c[t];
+  std::vector<double> q, r, full(L), c(n_lags);
+  inverse_psd(L, fs, sigma, fknee, alpha, q, r);
+  for (int k = -1; k < (dlags_out ? 3 : 0); ++k) {   // the lags, then their gradients
+    for (int j = 0; j <= L / 2; ++j) {
+      const double v = k < 0 ? q[j] : inverse_psd_grad(k, j, L, fs, sigma, fknee, alpha, q[j], r[j]);
+      full[j] = v;
+      if (j > 0) full[L - j] = v;
     }
+    even_idft(full, n_lags, c.data());
+    double* out = k < 0 ? lags_out : dlags_out + (size_t)k * n_lags;
+    for (int t = 0; t < n_lags; ++t) out[t] = (1.0 - (double)t / n_lags) * c[t];
   }
   return MADMAP_OK;
 }
 
+// The chain rule by the transposed transform: one transform of the tapered
+// gradient instead of one per parameter and one for the lags.
 extern "C" madmap_status madmap_noise_filter_vjp(int32_t n_lags, double fs, double sigma, double fknee, double alpha,
                                                  const double* grad_lags, double* grad_params_out) {
   MM_CHECK(n_lags >= 1 && grad_lags && grad_params_out, MADMAP_ERR_INVALID_ARG, "noise_filter_vjp: bad arguments");
-  std::vector<double> lags(n_lags), dl(3 * (size_t)n_lags);
-  madmap_status st = madmap_noise_filter(n_lags, fs, sigma, fknee, alpha, lags.data(), dl.data());
-  if (st != MADMAP_OK) return st;
+  MM_CHECK(fs > 0 && sigma > 0 && fknee >= 0 && isfinite(alpha), MADMAP_ERR_INVALID_ARG,
+           "noise_filter: need fs > 0, sigma > 0, fknee >= 0, finite alpha");
+  const int L = 4 * n_lags;
+  std::vector<double> q, r, h(n_lags), w(L / 2 + 1);
+  inverse_psd(L, fs, sigma, fknee, alpha, q, r);
+  for (int t = 0; t < n_lags; ++t) h[t] = (1.0 - (double)t / n_lags) * grad_lags[t];
+  even_idft_transpose(h.data(), n_lags, (size_t)L, w.data());
   for (int k = 0; k < 3; ++k) {
     double acc = 0.0;
-    for (int t = 0; t < n_lags; ++t) acc += dl[(size_t)k * n_lags + t] * grad_lags[t];
-    grad_params_out[k] = acc;
+    for (int j = 0; j <= L / 2; ++j)
+      acc += (j == 0 || j == L / 2 ? 1.0 : 2.0) * inverse_psd_grad(k, j, L, fs, sigma, fknee, alpha, q[j], r[j]) * w[j];
+    grad_params_out[k] = acc / (double)L;
   }
   return MADMAP_OK;
 }
