@@ -34,6 +34,7 @@
 #include <chrono>
 #include <climits>
 #include <cstring>
+#include <type_traits>
 #include <vector>
 
 #include "internal.cuh"
@@ -83,9 +84,16 @@ struct SolveBuffers {
   size_t bytes = 0;
 };
 
-static const int NB = 304;  // blocks of the vector kernels (2 per SM)
+// Blocks of the vector kernels (2 per SM; 4, 6, 8 and 16 measured the same or
+// slower: all-sky mixed solve 19.90, 19.90, 20.01, 20.15, 20.65 ms)
+static const int NB = 304;
 static const int HIST_CAP = 4096;  // iterations whose residual is recorded per right-hand side
 static const int NT = 256;
+
+static int grid_vec(long long n) {
+  long long g = (n + NT - 1) / NT;
+  return (int)std::max(1LL, std::min<long long>(g, NB));
+}
 
 static void free_one(SolveBuffers* sb) {
   if (!sb) return;
@@ -546,23 +554,44 @@ __global__ void __launch_bounds__(NT) k_cg_replace(Real* x, Real* r, Real* z, Re
 }
 
 // ---------------------------------------------------------------- layout and refinement kernels
-// user [n][ns] (U) -> padded working layout [n][ns_pad] (Real)
-template <typename U, typename Real>
-__global__ void k_pack(const U* in, Real* out, int n_obs, int ns, int ns_pad) {
-  const long long n = (long long)n_obs * ns_pad;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const int s = (int)(i % ns_pad);
-    const long long pp = i / ns_pad;
-    out[i] = s < ns ? (Real)in[pp * ns + s] : (Real)0;
+// user [n][ns] (U) -> padded working layout [n][ns_pad] (Real; df64: split into
+// pairs), one thread per row; zero (may be NULL) is cleared in the same pass.
+template <typename U, typename Real, typename Z>
+__global__ void __launch_bounds__(NT) k_pack(const U* __restrict__ in, Real* __restrict__ out, int n_obs, int ns,
+                                             Z* __restrict__ zero) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n_obs; i += gridDim.x * blockDim.x) {
+    if (ns == 1) {
+      out[i] = (Real)in[i];
+      if (zero) zero[i] = Z(0);
+      continue;
+    }
+    const U a = in[3LL * i], b = in[3LL * i + 1], c = in[3LL * i + 2];
+    if constexpr (std::is_same<Real, df64>::value) {
+      const df64 A((double)a), B((double)b), D((double)c);
+      float4* o = reinterpret_cast<float4*>(out) + 2LL * i;
+      o[0] = make_float4(A.hi, A.lo, B.hi, B.lo);
+      o[1] = make_float4(D.hi, D.lo, 0.f, 0.f);
+    } else {
+      const V3<Real, 3> v = {(Real)a, (Real)b, (Real)c};
+      stv<Real, 3>(out, i, v);
+    }
+    if (zero) {
+      const V3<Z, 3> v = {0, 0, 0};
+      stv<Z, 3>(zero, i, v);
+    }
   }
 }
 template <typename Real, typename U>
-__global__ void k_unpack(const Real* in, U* out, int n_obs, int ns, int ns_pad) {
-  const long long n = (long long)n_obs * ns;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const int s = (int)(i % ns);
-    const long long pp = i / ns;
-    out[i] = (U)in[pp * ns_pad + s];
+__global__ void __launch_bounds__(NT) k_unpack(const Real* __restrict__ in, U* __restrict__ out, int n_obs, int ns) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n_obs; i += gridDim.x * blockDim.x) {
+    if (ns == 1) {
+      out[i] = (U)in[i];
+      continue;
+    }
+    const V3<Real, 3> v = ldv<Real, 3>(in, i);
+    out[3LL * i] = (U)v.a;
+    out[3LL * i + 1] = (U)v.b;
+    out[3LL * i + 2] = (U)v.c;
   }
 }
 
@@ -633,10 +662,6 @@ __global__ void k_take_best(const double* x64, double* xbest64, long long nvec, 
     xbest64[o + i] = x64[o + i];
 }
 
-static int grid_vec(long long n) {
-  long long g = (n + NT - 1) / NT;
-  return (int)std::max(1LL, std::min<long long>(g, NB));
-}
 
 // ---------------------------------------------------------------- PCG driver
 struct Batch {
@@ -879,14 +904,14 @@ static madmap_status run_pcg(Plan* p, SolveBuffers* sb, const Batch& B, const Bt
 template <int NS>
 static madmap_status write_checkpoint(Plan* p, SolveBuffers* sb, const CgState& h, madmap_checkpoint* c,
                                       cudaStream_t s) {
-  const int n = p->n_obs, ns = p->n_stokes, np = p->ns_pad;
+  const int n = p->n_obs, ns = p->n_stokes;
   const long long user = (long long)n * ns;
   const double* src[5] = {(const double*)sb->x, (const double*)sb->r, (const double*)sb->z, (const double*)sb->p,
                           (const double*)sb->xb};
   double* dst[5] = {c->x, c->r, c->z, c->p, c->x_best};
   for (int k = 0; k < 5; ++k) {
     count_launches(1);
-    k_unpack<double, double><<<grid_vec(user), NT, 0, s>>>(src[k], sb->b64, n, ns, np);
+    k_unpack<double, double><<<grid_vec(n), NT, 0, s>>>(src[k], sb->b64, n, ns);
     MM_CUDA(cudaMemcpyAsync(dst[k], sb->b64, sizeof(double) * user, cudaMemcpyDeviceToHost, s));
   }
   MM_CUDA(cudaStreamSynchronize(s));
@@ -1233,8 +1258,8 @@ static madmap_status solve_impl(Plan* p, int n_rhs, const float* d, double* m, c
   if (st != MADMAP_OK) return st;
   for (int k = 0; k < n_rhs; ++k) {
     count_launches(1);
-    k_unpack<double, double><<<grid_vec((long long)n * p->n_stokes), NT, 0, s>>>(
-        xr + k * nv, m + (long long)k * n * p->n_stokes, n, p->n_stokes, p->ns_pad);
+    k_unpack<double, double><<<grid_vec(n), NT, 0, s>>>(xr + k * nv, m + (long long)k * n * p->n_stokes, n,
+                                                         p->n_stokes);
   }
   MM_CUDA(cudaStreamSynchronize(s));
   MM_CUDA(cudaGetLastError());
@@ -1253,14 +1278,14 @@ static madmap_status resume_impl(Plan* p, const madmap_checkpoint* c, double* m,
   SolveBuffers* sb = nullptr;
   madmap_status st = get_buffers(p, true, 1, &sb);
   if (st != MADMAP_OK) return st;
-  const int n = p->n_obs, ns = p->n_stokes, np = p->ns_pad;
+  const int n = p->n_obs, ns = p->n_stokes;
   const long long user = (long long)n * ns;
   const double* src[5] = {c->x, c->r, c->z, c->p, c->x_best};
   double* dst[5] = {(double*)sb->x, (double*)sb->r, (double*)sb->z, (double*)sb->p, (double*)sb->xb};
   for (int k = 0; k < 5; ++k) {
     MM_CUDA(cudaMemcpyAsync(sb->b64, src[k], sizeof(double) * user, cudaMemcpyHostToDevice, s));
     count_launches(1);
-    k_pack<double, double><<<grid_vec((long long)n * np), NT, 0, s>>>(sb->b64, dst[k], n, ns, np);
+    k_pack<double, double, double><<<grid_vec(n), NT, 0, s>>>(sb->b64, dst[k], n, ns, nullptr);
   }
   MM_CUDA(cudaMemsetAsync(sb->q, 0, sizeof(double) * sb->nvec, s));
   const int every = o.checkpoint_every > 0 ? o.checkpoint_every : 0;
@@ -1293,7 +1318,7 @@ static madmap_status resume_impl(Plan* p, const madmap_checkpoint* c, double* m,
     if ((st = append_hist(sb, 0, c->iters + 1, R[0].iters, 1.0, Hh[0], s)) != MADMAP_OK) return st;
   }
   count_launches(1);
-  k_unpack<double, double><<<grid_vec(user), NT, 0, s>>>((const double*)sb->xb, m, n, ns, np);
+  k_unpack<double, double><<<grid_vec(n), NT, 0, s>>>((const double*)sb->xb, m, n, ns);
   MM_CUDA(cudaStreamSynchronize(s));
   MM_CUDA(cudaGetLastError());
   std::vector<madmap_solve_info> Iv(1);
@@ -1463,7 +1488,7 @@ static madmap_status backward_impl(Plan* p, const float* d, const double* m, con
   }
   // adjoint solve H lambda = dL/dm (zero at excised pixels)
   count_launches(2);
-  k_pack<double, double><<<grid_vec(nv), NT, 0, s>>>(gm, sb64->b64, n, ns, np);
+  k_pack<double, double, double><<<grid_vec(n), NT, 0, s>>>(gm, sb64->b64, n, ns, nullptr);
   k_mask_excised<<<grid_vec(nv), NT, 0, s>>>(sb64->b64, n, np, p->excised, p->multires ? p->excised_pol : nullptr,
                                              p->ext ? (long long)p->n_obs_sky : (long long)n);
   std::vector<madmap_solve_info> I(1);
@@ -1478,7 +1503,7 @@ static madmap_status backward_impl(Plan* p, const float* d, const double* m, con
   k_unpoint<NS><<<std::max(1, gt), 256, 0, s>>>(lam, p->pix_obs, pix_pol, p->cs64, nullptr, 0.0, 1.0, p->bw_a, nt,
                                                 otf_pointing(p), p->ext_row, p->hwp_base, p->hwp_ang,
                                                 p->hwp_tau);
-  k_pack<double, double><<<grid_vec(nv), NT, 0, s>>>(m, sb64->t64, n, ns, np);
+  k_pack<double, double, double><<<grid_vec(n), NT, 0, s>>>(m, sb64->t64, n, ns, nullptr);
   k_unpoint<NS><<<std::max(1, gt), 256, 0, s>>>(sb64->t64, p->pix_obs, pix_pol, p->cs64, d, 1.0, -1.0, p->bw_r, nt,
                                                 otf_pointing(p), p->ext_row, p->hwp_base, p->hwp_ang,
                                                 p->hwp_tau);
@@ -1522,30 +1547,46 @@ static madmap_status backward_impl(Plan* p, const float* d, const double* m, con
 }
 
 // ---------------------------------------------------------------- operator entry points
+static bool disjoint(const void* a, long long na, const void* b, long long nb) {
+  const char *p = static_cast<const char*>(a), *q = static_cast<const char*>(b);
+  return p + na <= q || q + nb <= p;
+}
+
+// Temperature maps have the user's layout, so the operator reads and writes
+// the user's buffers directly (unless they overlap); IQU rows are padded to
+// four values on the way in and unpadded on the way out.
 template <typename Real>
 static madmap_status apply_impl(Plan* p, int prec, int n_rhs, const void* x, void* y, cudaStream_t s) {
   SolveBuffers* sb = nullptr;
   madmap_status st = get_buffers(p, prec != OPP_F32, 1, &sb);
   if (st != MADMAP_OK) return st;
-  const int n = p->n_obs, ns = p->n_stokes, np = p->ns_pad;
+  const int n = p->n_obs, ns = p->n_stokes;
   const long long user = (long long)n * ns;
+  const long long bytes = (long long)sizeof(Real) * user * n_rhs;
+  const bool direct = ns == 1 && disjoint(x, bytes, y, bytes);
   for (int r = 0; r < n_rhs; ++r) {
     const Real* xr = static_cast<const Real*>(x) + r * user;
     Real* yr = static_cast<Real*>(y) + r * user;
-    count_launches(2);
-    k_pack<Real, Real><<<grid_vec((long long)n * np), NT, 0, s>>>(xr, (Real*)sb->p, n, ns, np);
-    MM_CUDA(cudaMemsetAsync(sb->q, 0, sizeof(Real) * sb->nvec, s));
-    const void* xin = sb->p;
+    Real* q = direct ? yr : (Real*)sb->q;
+    const void* xin = direct ? (const void*)xr : sb->p;
     if (prec == OPP_DF64) {
       count_launches(1);
-      k_split<<<grid_vec(sb->nvec), NT, 0, s>>>((const double*)sb->p, sb->xdf, sb->nvec);
+      k_pack<Real, df64, Real><<<grid_vec(n), NT, 0, s>>>(xr, sb->xdf, n, ns, q);
       xin = sb->xdf;
+    } else if (direct) {
+      MM_CUDA(cudaMemsetAsync(q, 0, sizeof(Real) * user, s));
+    } else {
+      count_launches(1);
+      k_pack<Real, Real, Real><<<grid_vec(n), NT, 0, s>>>(xr, (Real*)sb->p, n, ns, q);
     }
-    st = op_launch(p, prec, IN_MAP, OUT_MAP, xin, sb->q, 0, 0, 1, nullptr, s);
+    st = op_launch(p, prec, IN_MAP, OUT_MAP, xin, q, 0, 0, 1, nullptr, s);
     if (st == MADMAP_OK)
-      st = reduce_across(p, sb->q, sb->nvec, prec == OPP_F32 ? MADMAP_REDUCE_F32 : MADMAP_REDUCE_F64, s);
+      st = reduce_across(p, q, sb->nvec, prec == OPP_F32 ? MADMAP_REDUCE_F32 : MADMAP_REDUCE_F64, s);
     if (st != MADMAP_OK) return st;
-    k_unpack<Real, Real><<<grid_vec(user), NT, 0, s>>>((const Real*)sb->q, yr, n, ns, np);
+    if (!direct) {
+      count_launches(1);
+      k_unpack<Real, Real><<<grid_vec(n), NT, 0, s>>>(q, yr, n, ns);
+    }
   }
   MM_CUDA(cudaGetLastError());
   return MADMAP_OK;
@@ -1556,17 +1597,21 @@ static madmap_status rhs_impl(Plan* p, int prec, int n_rhs, const float* d, void
   SolveBuffers* sb = nullptr;
   madmap_status st = get_buffers(p, prec != OPP_F32, 1, &sb);
   if (st != MADMAP_OK) return st;
-  const int n = p->n_obs, ns = p->n_stokes, np = p->ns_pad;
+  const int n = p->n_obs, ns = p->n_stokes;
   const long long user = (long long)n * ns;
+  const bool direct = ns == 1 && disjoint(d, (long long)sizeof(float) * p->n_t * n_rhs, b,
+                                          (long long)sizeof(Real) * user * n_rhs);
   for (int r = 0; r < n_rhs; ++r) {
-    MM_CUDA(cudaMemsetAsync(sb->q, 0, sizeof(Real) * sb->nvec, s));
-    st = op_launch(p, prec, IN_TOD, OUT_MAP, d + (long long)r * p->n_t, sb->q, 0, 0, 1, nullptr, s);
+    Real* const br = static_cast<Real*>(b) + r * user;
+    Real* const q = direct ? br : (Real*)sb->q;
+    MM_CUDA(cudaMemsetAsync(q, 0, sizeof(Real) * sb->nvec, s));
+    st = op_launch(p, prec, IN_TOD, OUT_MAP, d + (long long)r * p->n_t, q, 0, 0, 1, nullptr, s);
     if (st == MADMAP_OK)
-      st = reduce_across(p, sb->q, sb->nvec, prec == OPP_F32 ? MADMAP_REDUCE_F32 : MADMAP_REDUCE_F64, s);
+      st = reduce_across(p, q, sb->nvec, prec == OPP_F32 ? MADMAP_REDUCE_F32 : MADMAP_REDUCE_F64, s);
     if (st != MADMAP_OK) return st;
+    if (direct) continue;
     count_launches(1);
-    k_unpack<Real, Real><<<grid_vec(user), NT, 0, s>>>((const Real*)sb->q, static_cast<Real*>(b) + r * user, n, ns,
-                                                       np);
+    k_unpack<Real, Real><<<grid_vec(n), NT, 0, s>>>(q, br, n, ns);
   }
   MM_CUDA(cudaGetLastError());
   return MADMAP_OK;
