@@ -20,7 +20,8 @@ CSRC = os.path.join(PKG, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(ROOT, "_build")
 LIB = os.path.join(PKG, "libmadmap.so")
-SOURCES = ["plan.cu", "operator.cu", "operator_f32.cu", "operator_f64.cu", "operator_df64.cu", "solver.cu"]
+SOURCES = ["plan.cu", "operator.cu", "operator_f32.cu", "operator_f64.cu", "operator_df64.cu", "solver.cu",
+           "spectra.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

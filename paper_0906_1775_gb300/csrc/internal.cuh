@@ -276,7 +276,19 @@ inline int reg_log_n1(int M) { return (M >= (1 << 14) && M <= (1 << 18)) ? __bui
 size_t reg_table_floats(int logN1);
 void reg_fill_tables(int logN1, float* out);
 RegTables reg_point_tables(int logN1, const float* base);
-void reg_spectrum(const std::vector<double>& re, int logN1, float* h32);
+
+// Lag correlation of the backward pass by transforms (spectra.cu): windows of
+// length M in pairs, each pair twice (a, then r), and the cross spectra.
+struct CorrPlan {
+  int M = 0, logN1 = 0, logN2 = 0;
+  RegTables reg;
+  const double2* tw = nullptr;   // [M]
+  Tile* tiles = nullptr;         // [2 n_pairs]
+  int n_pairs = 0, per_chunk = 0;
+  void* scratch = nullptr;
+  size_t scratch_bytes = 0;
+  double* G = nullptr;           // [n_filters][256][M / 256]; NULL until set up
+};
 
 // ---------------------------------------------------------------- plan
 struct SolveBuffers;  // solver.cu
@@ -381,8 +393,8 @@ struct Plan {
   cudaEvent_t solve_event = nullptr;
   std::vector<TileSet*> tile_sets;  // batched tile lists by n_rhs (device memory in allocs)
   // backward pass: timestreams A lambda and d - A m, lag-correlation work items
-  float* bw_a = nullptr;
-  float* bw_r = nullptr;
+  float* bw_a = nullptr;           // [2 n_t]: a, then r
+  CorrPlan corr;
   void* corr_items = nullptr;
   int n_corr_items = 0;
   // deterministic plans: the samples of every observed row in ascending order
@@ -503,7 +515,17 @@ madmap_status get_tile_set(Plan* p, int n_rhs, TileSet** out);
 // Deterministic plans: a timestream buffer for n_rhs right-hand sides.
 madmap_status ensure_wtod(Plan* p, int n_rhs);
 
-// host FFT (radix 2, float64), used at plan time only
+// Spectra of p->lags into H64, H32, Hdf on the device (spectra.cu); waits for s.
+madmap_status build_spectra(Plan* p, cudaStream_t s);
+
+// Backward pass: lag correlation of p->bw_a by transforms where corr_by_fft;
+// corr_spectrum (operator_f32.cu) sums the windows' cross spectra into corr.G.
+bool corr_by_fft(const Plan* p);
+madmap_status corr_setup(Plan* p, cudaStream_t s);
+madmap_status corr_spectrum(Plan* p, cudaStream_t s);
+madmap_status corr_run(Plan* p, double* grad, cudaStream_t s);
+
+// host FFT (radix 2, float64), for the noise filters and the allocation-free weighting
 void host_fft(std::vector<double>& re, std::vector<double>& im, bool inverse);
 
 // ---------------------------------------------------------------- device helpers

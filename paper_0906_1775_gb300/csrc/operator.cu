@@ -133,6 +133,14 @@ madmap_status noalloc_scratch(void** out) {
   return MADMAP_OK;
 }
 
+// The spectrum re (length 256 N1) as the register kernels read it: [k2][k1], / M.
+void reg_spectrum(const std::vector<double>& re, int logN1, float* h32) {
+  const int N1 = 1 << logN1;
+  const double M = (double)REG_N2 * N1;
+  for (int k2 = 0; k2 < REG_N2; ++k2)
+    for (int k1 = 0; k1 < N1; ++k1) h32[(size_t)k2 * N1 + k1] = (float)(re[k2 + (size_t)REG_N2 * k1] / M);
+}
+
 size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
 
 }  // namespace

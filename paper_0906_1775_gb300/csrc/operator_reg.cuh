@@ -331,6 +331,59 @@ __global__ void __launch_bounds__(256, MM_MINB_C3) k_c3(OpArgs a) {
   }
 }
 
+// ---------------------------------------------------------------- k_xcorr
+// Backward pass: row transforms of a window pair's a and r (scratch tiles 2 i
+// and 2 i + 1, from k_c1) and their cross spectrum Re(conj(Z_a) Z_r), added in
+// float64 to the filter's G [k2][k1].
+template <int LA, int LB>
+__device__ __forceinline__ void row_forward(const float2* sc, float2* x, const float4* row, int l,
+                                            float2 (&z)[1 << LA]) {
+  typedef RowGeom<LA, LB> G;
+  constexpr int RA = G::RA, RB = G::RB, Q = RA / RB;
+  float2 v[RA];
+#pragma unroll
+  for (int u = 0; u < RA; ++u) v[u] = sc[RB * u];
+  reg_dft<LA, false>(v);
+  const Powers<LA> w(row + 4 * l);
+  __syncwarp();
+#pragma unroll
+  for (int m = 0; m < RA; ++m) {
+    const int p = brev_lg<LA>(m);
+    x[p * G::S + l] = p == 0 ? v[m] : cmul(v[m], w(p));
+  }
+  __syncwarp();
+#pragma unroll
+  for (int q = 0; q < Q; ++q) {
+    float2 t[RB];
+#pragma unroll
+    for (int m = 0; m < RB; ++m) t[m] = x[(l + RB * q) * G::S + m];
+    reg_dft<LB, false>(t);
+#pragma unroll
+    for (int m = 0; m < RB; ++m) z[q * RB + brev_lg<LB>(m)] = t[m];
+  }
+}
+template <int LA, int LB>
+__global__ void __launch_bounds__(128, LA == 5 ? 2 : 4) k_xcorr(OpArgs a, double* G0) {
+  typedef RowGeom<LA, LB> G;
+  constexpr int RA = G::RA, RB = G::RB, Q = RA / RB, LN = LA + LB;
+  __shared__ float2 buf[G::ROWS * G::ROW];
+  const int l = threadIdx.x & (RB - 1), r = threadIdx.x / RB;
+  const int row = blockIdx.x * G::ROWS + r;
+  const int filt = a.tiles[a.tile0 + 2 * blockIdx.y].filter;
+  const float2* sc = static_cast<const float2*>(a.scratch) + 2LL * blockIdx.y * a.M + ((long long)row << LN) + l;
+  float2 za[RA], zr[RA];
+  row_forward<LA, LB>(sc, buf + r * G::ROW, a.reg_row, l, za);
+  row_forward<LA, LB>(sc + a.M, buf + r * G::ROW, a.reg_row, l, zr);
+  double* g = G0 + (long long)filt * a.M + ((long long)row << LN) + l;
+#pragma unroll
+  for (int q = 0; q < Q; ++q)
+#pragma unroll
+    for (int b = 0; b < RB; ++b) {
+      const float2 u = za[q * RB + b], v = zr[q * RB + b];
+      atomicAdd(g + RB * q + RA * b, (double)u.x * (double)v.x + (double)u.y * (double)v.y);
+    }
+}
+
 // The kernels of a plan with register transforms, and their grids for nt tiles.
 template <int NS, int IN, int OUT>
 inline void launch_reg(const OpArgs& a, int nt, cudaStream_t s, cudaEvent_t* ev, int* ei) {

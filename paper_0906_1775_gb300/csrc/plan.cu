@@ -7,10 +7,8 @@
 #include <stdlib.h>
 
 #include <algorithm>
-#include <atomic>
 #include <cstring>
 #include <string>
-#include <thread>
 #include <vector>
 
 #include "internal.cuh"
@@ -1100,77 +1098,6 @@ RegTables reg_point_tables(int logN1, const float* base) {
   return t;
 }
 
-// The spectrum re (length 256 N1) as the register kernels read it: [k2][k1], / M.
-void reg_spectrum(const std::vector<double>& re, int logN1, float* h32) {
-  const int N1 = 1 << logN1;
-  const double M = (double)REG_N2 * N1;
-  for (int k2 = 0; k2 < REG_N2; ++k2)
-    for (int k1 = 0; k1 < N1; ++k1) h32[(size_t)k2 * N1 + k1] = (float)(re[k2 + (size_t)REG_N2 * k1] / M);
-}
-
-// Spectrum of one filter's circulant embedding into h64/h32/hdf (the layout
-// the row kernel reads); returns false when the symbol is not positive.
-static bool filter_spectrum(const Plan* p, int f, double* h64, float* h32, df64* hdf, double* min_out) {
-  const int M = p->M;
-  std::vector<double> re(M, 0.0), im(M, 0.0);
-  const double* lg = &p->lags[(size_t)f * p->n_lags];
-  re[0] = lg[0];
-  for (int t = 1; t < p->n_lags; ++t) {
-    re[t] += lg[t];
-    re[M - t] += lg[t];
-  }
-  host_fft(re, im, false);
-  double mn = 1e300;
-  for (int k = 0; k < M; ++k) mn = std::min(mn, re[k]);
-  *min_out = mn;
-  if (!(mn > 0.0)) return false;
-  for (int pos2 = 0; pos2 < p->N2; ++pos2) {
-    int k2 = 0;
-    for (int b = 0; b < p->logN2; ++b) k2 |= ((pos2 >> b) & 1) << (p->logN2 - 1 - b);
-    for (int pos1 = 0; pos1 < p->N1; ++pos1) {
-      int k1 = 0;
-      for (int b = 0; b < p->logN1; ++b) k1 |= ((pos1 >> b) & 1) << (p->logN1 - 1 - b);
-      const double v = re[k2 + (size_t)p->N2 * k1] / (double)M;
-      const size_t o = (size_t)pos2 * p->N1 + pos1;
-      h64[o] = v;
-      h32[o] = (float)v;
-      hdf[o] = df64(v);
-    }
-  }
-  if (p->reg.logN1 > 0) reg_spectrum(re, p->reg.logN1, h32);
-  return true;
-}
-
-// All filters' spectra, computed on host threads (one filter per task).
-static madmap_status build_spectra(Plan* p) {
-  const int M = p->M, F = p->n_filters;
-  std::vector<double> h64((size_t)F * M);
-  std::vector<float> h32((size_t)F * M);
-  std::vector<df64> hdf((size_t)F * M);
-  std::vector<double> mins(F, 0.0);
-  std::vector<char> ok(F, 0);
-  const int T = std::max(1, std::min<int>(F, (int)std::max(1u, std::thread::hardware_concurrency())));
-  std::atomic<int> next(0);
-  auto work = [&]() {
-    for (int f = next++; f < F; f = next++)
-      ok[f] = filter_spectrum(p, f, &h64[(size_t)f * M], &h32[(size_t)f * M], &hdf[(size_t)f * M], &mins[f]);
-  };
-  std::vector<std::thread> pool;
-  for (int t = 1; t < T; ++t) pool.emplace_back(work);
-  work();
-  for (auto& th : pool) th.join();
-  for (int f = 0; f < F; ++f)
-    if (!ok[f]) {
-      set_error("filter " + std::to_string(f) + " is not positive definite (circulant symbol minimum " +
-                std::to_string(mins[f]) + ")");
-      return MADMAP_ERR_NOT_PD;
-    }
-  MM_CUDA(cudaMemcpy(p->H64, h64.data(), h64.size() * sizeof(double), cudaMemcpyHostToDevice));
-  MM_CUDA(cudaMemcpy(p->H32, h32.data(), h32.size() * sizeof(float), cudaMemcpyHostToDevice));
-  MM_CUDA(cudaMemcpy(p->Hdf, hdf.data(), hdf.size() * sizeof(df64), cudaMemcpyHostToDevice));
-  return MADMAP_OK;
-}
-
 // Multi-resolution preconditioner and classification.  Every call passes over
 // the samples (no per-filter sums are kept); the first also stores the
 // float64 weights, zeroes the rows of excised Q/U pixels and packs the
@@ -1441,7 +1368,6 @@ static madmap_status setup_windows(Plan* p, int M, long long tpc_req, cudaStream
     MM_CUDA(cudaMemcpy(tab, h.data(), sizeof(float) * h.size(), cudaMemcpyHostToDevice));
     p->reg = reg_point_tables(rl, tab);
   }
-  if ((st = build_spectra(p)) != MADMAP_OK) return st;
   {
     std::vector<double2> t64(p->M);
     std::vector<float2> t32(p->M);
@@ -1465,7 +1391,8 @@ static madmap_status setup_windows(Plan* p, int M, long long tpc_req, cudaStream
     p->scratch_slots = n_chunks > 1 ? 2 : 1;
     if (n_chunks > 1 && (st = ensure_op_streams(p)) != MADMAP_OK) return st;
   }
-  return walloc(p, &p->scratch, (size_t)p->scratch_slots * p->tiles_per_chunk * p->M * sizeof(double2));
+  st = walloc(p, &p->scratch, (size_t)p->scratch_slots * p->tiles_per_chunk * p->M * sizeof(double2));
+  return st == MADMAP_OK ? build_spectra(p, s) : st;
 }
 
 // Plans whose column kernels can sum runs of one pixel before the scatter's
@@ -2054,10 +1981,13 @@ extern "C" madmap_status madmap_plan_set_filters(madmap_plan_t plan, const doubl
     MM_CHECK(isfinite(lags[k]), MADMAP_ERR_INVALID_ARG, "filter_lags must be finite");
   std::vector<double> old = p->lags;
   p->lags.assign(lags, lags + (size_t)p->n_filters * p->n_lags);
-  madmap_status st = build_spectra(p);
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  madmap_status st = build_spectra(p, s);
   if (st != MADMAP_OK) {
+    const std::string why = madmap_last_error();
     p->lags = old;
-    build_spectra(p);
+    build_spectra(p, s);
+    set_error(why);
     return st;
   }
   if (p->diag) {  // the white-noise pass reads f(0) directly
@@ -2066,6 +1996,5 @@ extern "C" madmap_status madmap_plan_set_filters(madmap_plan_t plan, const doubl
   // The block preconditioner weighs samples by f(0) of their filter: rebuild it.
   // Rows of excised pixels are already zero, so those pixels have no hits and
   // classify as excised again; every other pixel keeps its A^T A block.
-  cudaStream_t s = static_cast<cudaStream_t>(stream);
   return build_preconditioner(p, s);
 }

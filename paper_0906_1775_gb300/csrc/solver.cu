@@ -1392,7 +1392,8 @@ __global__ void k_mask_excised(double* b, long long nvec_pixels, int ns_pad, con
   }
 }
 
-// Lag correlation sum_{|t-t'|=tau} a_t r_t' by direct sums: CTA (lag block,
+// Lag correlation sum_{|t-t'|=tau} a_t r_t' by direct sums, for more lags than
+// the transforms of spectra.cu take windows for (corr_by_fft): CTA (lag block,
 // work item) covers CORR_LB lags over the samples [t_lo, t_hi) of one
 // interval, in tiles of CORR_TT samples staged in shared memory, and adds
 // its totals to grad[filter][tau] (float64 atomics, one per lag and item).
@@ -1482,10 +1483,10 @@ static madmap_status backward_impl(Plan* p, const float* d, const double* m, con
   const int n = p->n_obs, ns = p->n_stokes, np = p->ns_pad;
   const long long nt = p->n_t;
   if (!p->bw_a) {
-    st = dalloc_t(p, &p->bw_a, std::max(1LL, nt));
-    if (st == MADMAP_OK) st = dalloc_t(p, &p->bw_r, std::max(1LL, nt));
+    st = dalloc_t(p, &p->bw_a, std::max(1LL, 2 * nt));
     if (st != MADMAP_OK) return st;
   }
+  float* const bw_r = p->bw_a + nt;
   // adjoint solve H lambda = dL/dm (zero at excised pixels)
   count_launches(2);
   k_pack<double, double, double><<<grid_vec(n), NT, 0, s>>>(gm, sb64->b64, n, ns, nullptr);
@@ -1504,14 +1505,16 @@ static madmap_status backward_impl(Plan* p, const float* d, const double* m, con
                                                 otf_pointing(p), p->ext_row, p->hwp_base, p->hwp_ang,
                                                 p->hwp_tau);
   k_pack<double, double, double><<<grid_vec(n), NT, 0, s>>>(m, sb64->t64, n, ns, nullptr);
-  k_unpoint<NS><<<std::max(1, gt), 256, 0, s>>>(sb64->t64, p->pix_obs, pix_pol, p->cs64, d, 1.0, -1.0, p->bw_r, nt,
+  k_unpoint<NS><<<std::max(1, gt), 256, 0, s>>>(sb64->t64, p->pix_obs, pix_pol, p->cs64, d, 1.0, -1.0, bw_r, nt,
                                                 otf_pointing(p), p->ext_row, p->hwp_base, p->hwp_ang,
                                                 p->hwp_tau);
   if (grad_d) {
     st = op_launch(p, false, IN_TOD_REAL, OUT_TOD, p->bw_a, grad_d, 0, 0, 1, nullptr, s);
     if (st != MADMAP_OK) return st;
   }
-  if (grad_lags) {
+  if (grad_lags && corr_by_fft(p)) {
+    if ((st = corr_setup(p, s)) != MADMAP_OK || (st = corr_run(p, grad_lags, s)) != MADMAP_OK) return st;
+  } else if (grad_lags) {
     if (!p->corr_items) {
       std::vector<CorrItem> items;
       const long long chunk = 65536;
@@ -1532,9 +1535,11 @@ static madmap_status backward_impl(Plan* p, const float* d, const double* m, con
     for (int y0 = 0; y0 < p->n_corr_items; y0 += 65535) {
       const int ny = std::min(65535, p->n_corr_items - y0);
       count_launches(1);
-      k_lag_corr<<<dim3((p->n_lags + CORR_LB - 1) / CORR_LB, ny), CORR_T, 0, s>>>(p->bw_a, p->bw_r, items + y0,
+      k_lag_corr<<<dim3((p->n_lags + CORR_LB - 1) / CORR_LB, ny), CORR_T, 0, s>>>(p->bw_a, bw_r, items + y0,
                                                                                  p->n_lags, grad_lags);
     }
+  }
+  if (grad_lags) {
     st = reduce_across(p, grad_lags, (long long)p->n_filters * p->n_lags, MADMAP_REDUCE_F64, s);
     if (st != MADMAP_OK) return st;
   }

@@ -1,0 +1,313 @@
+// Float64 transforms of whole real sequences on the device: the filters'
+// spectra when a plan is built or its filters change, and the way back from
+// the backward pass's cross spectrum to lags.
+//
+// One complex FFT of length M = N1 N2 per filter in two kernels (columns, then
+// rows), with the shared-memory passes of the operator kernels.  Both
+// sequences are real and even up to what the caller drops, so only real parts
+// leave the second kernel.  (Two filters in one complex transform would let the
+// rounding of a large one into a much smaller one.)
+//
+// On the host the same transforms took 3.2 ms for 8 filters of M = 2^16 on 16
+// cores, most of a set_filters call; they are latency-bound here (two launches
+// of M / 2048 CTAs per filter, about 10^8 float64 operations).
+#include <math.h>
+
+#include <algorithm>
+#include <cstring>
+#include <string>
+#include <vector>
+
+#include "internal.cuh"
+
+namespace mm {
+
+namespace {
+
+// SPEC: x(n) = the circulant embedding of filter f's lags, out: H64, Hdf and
+// H32 / M in the operator kernels' order.  CORR: x(k) = the cross spectrum G
+// [k mod 256][k / 256], out: the correlations at lags 0 .. n_lags - 1.
+enum { SPEC = 0, CORR = 1 };
+struct SpecArgs {
+  int M, logN1, logN2, logB1, logB2, n_lags;
+  const double* x;
+  const double2* tw;   // [M] exp(-2 pi i j / M)
+  double2* scratch;    // [filters of the launch][M]
+  double* H64;
+  float* H32;
+  df64* Hdf;
+  int reg_logN1;       // SPEC: H32 in the register kernels' order; CORR: G's row length
+  unsigned long long* mins;  // SPEC: order-preserving bits of each filter's spectrum minimum
+  double* grad;
+};
+
+__device__ __forceinline__ unsigned long long order_bits(double v) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+  return (b >> 63) ? ~b : (b | 0x8000000000000000ull);
+}
+
+template <int MODE>
+__global__ void __launch_bounds__(OP_THREADS) k_spec_cols(SpecArgs a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  double2* buf = reinterpret_cast<double2*>(smem_raw);
+  const int N1 = 1 << a.logN1, B1 = 1 << a.logB1, rs = lay_rs(16, a.logN2, true);
+  constexpr int SW = 0;
+  double2* tw = buf + B1 * rs;
+  build_pass_twiddles(tw, a.logN2, a.tw, N1);
+  const int f = blockIdx.y, n1_0 = blockIdx.x * B1, total = B1 << a.logN2;
+  for (int e = threadIdx.x; e < total; e += OP_THREADS) {
+    const int n = n1_0 + (e & (B1 - 1)) + ((e >> a.logB1) << a.logN1);
+    double v;
+    if (MODE == SPEC) {
+      const int t = n < a.M - n ? n : a.M - n;
+      v = t < a.n_lags ? a.x[(long long)f * a.n_lags + t] : 0.0;
+    } else {
+      v = a.x[(long long)f * a.M + ((long long)(n & (REG_N2 - 1)) << a.reg_logN1) + (n >> 8)];
+    }
+    buf[(e & (B1 - 1)) * rs + swz<SW>(e >> a.logB1)] = make_double2(v, 0.0);
+  }
+  __syncthreads();
+  fft_rows<double2, false, SW>(buf, B1, rs, a.logN2, tw);
+  double2* sc = a.scratch + (long long)f * a.M;
+  for (int e = threadIdx.x; e < total; e += OP_THREADS) {
+    const int j = e & (B1 - 1), pos = e >> a.logB1;
+    const double2 w = a.tw[((n1_0 + j) * brev_n(pos, a.logN2)) & (a.M - 1)];
+    sc[((long long)pos << a.logN1) + n1_0 + j] = cmul(buf[j * rs + swz<SW>(pos)], w);
+  }
+}
+
+template <int MODE>
+__global__ void __launch_bounds__(OP_THREADS) k_spec_rows(SpecArgs a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  double2* buf = reinterpret_cast<double2*>(smem_raw);
+  const int N1 = 1 << a.logN1, B2 = 1 << a.logB2, rs = lay_rs(16, a.logN1, false);
+  constexpr int SW = 1;
+  double2* tw = buf + B2 * rs;
+  build_pass_twiddles(tw, a.logN1, a.tw, 1 << a.logN2);
+  const int f = blockIdx.y, pos0 = blockIdx.x * B2, total = B2 << a.logN1;
+  const double2* sc = a.scratch + (long long)f * a.M + ((long long)pos0 << a.logN1);
+  for (int e = threadIdx.x; e < total; e += OP_THREADS)
+    buf[(e >> a.logN1) * rs + swz<SW>(e & (N1 - 1))] = sc[e];
+  __syncthreads();
+  fft_rows<double2, false, SW>(buf, B2, rs, a.logN1, tw);
+  const double inv = 1.0 / (double)a.M;   // a power of two
+  unsigned long long mn = ~0ull;
+  for (int e = threadIdx.x; e < total; e += OP_THREADS) {
+    const int pos2 = pos0 + (e >> a.logN1), pos1 = e & (N1 - 1);
+    const double v = buf[(e >> a.logN1) * rs + swz<SW>(pos1)].x * inv;
+    const int k = brev_n(pos2, a.logN2) + (brev_n(pos1, a.logN1) << a.logN2);
+    if (MODE == SPEC) {
+      // a NaN orders above +inf as positive, so it is mapped below every value
+      const unsigned long long b = v == v ? order_bits(v) : 0ull;
+      mn = b < mn ? b : mn;
+      const long long o = (long long)f * a.M + ((long long)pos2 << a.logN1) + pos1;
+      a.H64[o] = v;
+      a.Hdf[o] = df64((float)v, (float)(v - (double)(float)v));
+      const long long r = a.reg_logN1 > 0
+                              ? (long long)f * a.M + ((long long)(k & (REG_N2 - 1)) << a.reg_logN1) + (k >> 8)
+                              : o;
+      a.H32[r] = (float)v;
+    } else if (k < a.n_lags) {
+      // c(tau) + c(-tau) = sum_k 2 G cos / M; tau = 0 counts once
+      a.grad[(long long)f * a.n_lags + k] = k == 0 ? v : 2.0 * v;
+    }
+  }
+  if (MODE == SPEC) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const unsigned long long b = __shfl_xor_sync(0xffffffffu, mn, o);
+      mn = b < mn ? b : mn;
+    }
+    if ((threadIdx.x & 31) == 0) atomicMin(a.mins + f, mn);
+  }
+}
+
+__global__ void k_fill_twiddles(double2* tw, int M) {
+  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < M; j += gridDim.x * blockDim.x) {
+    double s, c;
+    sincospi(2.0 * (double)j / (double)M, &s, &c);
+    tw[j] = make_double2(c, -s);
+  }
+}
+
+// Both kernels over n_f filters, at most `batch` (filters of scratch) a launch.
+template <int MODE>
+madmap_status run_spec(SpecArgs a, int n_f, int batch, cudaStream_t s) {
+  const int lg = a.logN1 + a.logN2, E = 11;   // 2048 elements per CTA
+  a.logB1 = std::max(0, std::min(E - a.logN2, a.logN1));
+  a.logB2 = std::max(0, std::min(E - a.logN1, a.logN2));
+  const size_t s1 = (((size_t)lay_rs(16, a.logN2, true) << a.logB1) + ((size_t)1 << a.logN2)) * 16;
+  const size_t s2 = (((size_t)lay_rs(16, a.logN1, false) << a.logB2) + ((size_t)1 << a.logN1)) * 16;
+  MM_CUDA(cudaFuncSetAttribute(k_spec_cols<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 << 10));
+  MM_CUDA(cudaFuncSetAttribute(k_spec_rows<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 << 10));
+  MM_CHECK(s1 <= (96u << 10) && s2 <= (96u << 10) && lg <= 20, MADMAP_ERR_INTERNAL, "spectra: bad geometry");
+  const SpecArgs b = a;
+  batch = std::min(batch, 65535);
+  for (int f = 0; f < n_f; f += batch) {
+    const int n = std::min(batch, n_f - f);
+    a.x = b.x + (MODE == SPEC ? (long long)f * a.n_lags : (long long)f * a.M);
+    if (MODE == SPEC) {
+      a.H64 = b.H64 + (long long)f * a.M;
+      a.H32 = b.H32 + (long long)f * a.M;
+      a.Hdf = b.Hdf + (long long)f * a.M;
+      a.mins = b.mins + f;
+    } else {
+      a.grad = b.grad + (long long)f * a.n_lags;
+    }
+    k_spec_cols<MODE><<<dim3(1 << (a.logN1 - a.logB1), n), OP_THREADS, s1, s>>>(a);
+    k_spec_rows<MODE><<<dim3(1 << (a.logN2 - a.logB2), n), OP_THREADS, s2, s>>>(a);
+    count_launches(2);
+  }
+  MM_CUDA(cudaGetLastError());
+  return MADMAP_OK;
+}
+
+}  // namespace
+
+// The spectra of all filters (p->lags) into p->H64, p->H32 and p->Hdf, using
+// p->tw64 and p->scratch; waits for the stream and fails when a symbol is not
+// positive.
+madmap_status build_spectra(Plan* p, cudaStream_t s) {
+  const int F = p->n_filters;
+  const size_t nl = p->lags.size();
+  // one temporary: lags, then the minima
+  double* dl = nullptr;
+  MM_CUDA(cudaMalloc(&dl, sizeof(double) * (nl + F)));
+  unsigned long long* mins = reinterpret_cast<unsigned long long*>(dl + nl);
+  std::vector<unsigned long long> h(F, ~0ull);
+  cudaError_t e = cudaMemcpyAsync(dl, p->lags.data(), sizeof(double) * nl, cudaMemcpyHostToDevice, s);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(mins, h.data(), sizeof(h[0]) * F, cudaMemcpyHostToDevice, s);
+  madmap_status st = e == cudaSuccess ? MADMAP_OK : cuda_fail(e, "cudaMemcpy (lags)");
+  if (st == MADMAP_OK) {
+    SpecArgs a = {};
+    a.M = p->M;
+    a.logN1 = p->logN1;
+    a.logN2 = p->logN2;
+    a.n_lags = p->n_lags;
+    a.x = dl;
+    a.tw = p->tw64;
+    a.scratch = static_cast<double2*>(p->scratch);
+    a.H64 = p->H64;
+    a.H32 = p->H32;
+    a.Hdf = p->Hdf;
+    a.reg_logN1 = p->reg.logN1;
+    a.mins = mins;
+    st = run_spec<SPEC>(a, F, p->scratch_slots * p->tiles_per_chunk, s);
+  }
+  if (st == MADMAP_OK) {
+    e = cudaMemcpyAsync(h.data(), mins, sizeof(h[0]) * F, cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e != cudaSuccess) st = cuda_fail(e, "spectra");
+  }
+  cudaFree(dl);
+  if (st != MADMAP_OK) return st;
+  for (int f = 0; f < F; ++f) {
+    const unsigned long long b = h[f];
+    double mn = NAN;
+    if (b != 0ull) {
+      const unsigned long long u = (b >> 63) ? (b & 0x7fffffffffffffffull) : ~b;
+      memcpy(&mn, &u, sizeof(mn));
+      mn *= (double)p->M;
+    }
+    if (!(mn > 0.0)) {
+      set_error("filter " + std::to_string(f) + " is not positive definite (circulant symbol minimum " +
+                std::to_string(mn) + ")");
+      return MADMAP_ERR_NOT_PD;
+    }
+  }
+  return MADMAP_OK;
+}
+
+// ---------------------------------------------------------------- lag correlation of the backward pass
+// sum_{|t - t'| = tau} a_t r_t' per filter for tau < n_lags, by transforms: in
+// each overlap-save window, a at the window's exact outputs and r over its
+// whole input have the wanted circular correlations at +-tau, so the cross
+// spectra Re(conj(Z_a) Z_r) of all windows of a filter are summed (float64) and
+// one float64 transform per filter returns the lags.  Two windows share a
+// complex transform: of conj(A + iA') (R + iR') the part that mixes them is odd
+// in k after taking the real part and leaves the (even) cosine sum unchanged.
+static constexpr int CORR_MAX_LAGS = 3 << 15;
+static constexpr size_t CORR_SCRATCH = (size_t)128 << 20;
+
+bool corr_by_fft(const Plan* p) { return p->n_lags <= CORR_MAX_LAGS; }
+
+madmap_status corr_setup(Plan* p, cudaStream_t s) {
+  CorrPlan& c = p->corr;
+  if (c.G) return MADMAP_OK;
+  madmap_status st = MADMAP_OK;
+  // the plan's own window length where it has register transforms, else the
+  // shortest one whose windows are at least half exact (a quarter at most lags)
+  int M = p->M;
+  const bool own = reg_log_n1(M) == 0;
+  if (own) {
+    M = 1 << 14;
+    while (M < (1 << 18) && M < 4 * p->n_lags) M <<= 1;
+  }
+  c.M = M;
+  const int rl = reg_log_n1(M), lg = rl + 8;
+  c.logN2 = (lg + 1) / 2;
+  c.logN1 = lg - c.logN2;
+  if (own) {
+    std::vector<float> h(reg_table_floats(rl));
+    reg_fill_tables(rl, h.data());
+    float* tab = nullptr;
+    if ((st = dalloc_t(p, &tab, h.size())) != MADMAP_OK) return st;
+    MM_CUDA(cudaMemcpy(tab, h.data(), sizeof(float) * h.size(), cudaMemcpyHostToDevice));
+    c.reg = reg_point_tables(rl, tab);
+    double2* tw = nullptr;
+    if ((st = dalloc_t(p, &tw, M)) != MADMAP_OK) return st;
+    k_fill_twiddles<<<(M + 255) / 256, 256, 0, s>>>(tw, M);
+    c.tw = tw;
+  } else {
+    c.reg = p->reg;
+    c.tw = p->tw64;
+  }
+  // window pairs, each twice: a at the exact outputs (rhs 0), r over the input (rhs 1)
+  std::vector<Tile> tiles, both;
+  build_tiles(p->offsets, p->ivl_filter, p->n_filters, p->n_lags, M, tiles);
+  for (const Tile& t : tiles) {
+    Tile ta = t, tr = t;
+    for (int l = 0; l < 2; ++l) {
+      ta.l[l].lo = t.l[l].ws + t.l[l].out_lo;
+      ta.l[l].hi = t.l[l].ws + t.l[l].out_hi;
+      ta.l[l].rhs = 0;
+      tr.l[l].rhs = 1;
+    }
+    both.push_back(ta);
+    both.push_back(tr);
+  }
+  c.n_pairs = (int)tiles.size();
+  c.per_chunk = (int)std::max<long long>(
+      1, std::min<long long>(std::min<long long>(c.n_pairs, 32767), (long long)(CORR_SCRATCH / (2 * (size_t)M * sizeof(float2)))));
+  if ((st = dalloc_t(p, &c.tiles, std::max<size_t>(1, both.size()))) != MADMAP_OK) return st;
+  if (!both.empty())
+    MM_CUDA(cudaMemcpy(c.tiles, both.data(), sizeof(Tile) * both.size(), cudaMemcpyHostToDevice));
+  // one buffer for the windows' transforms and then the float64 ones
+  c.scratch_bytes = std::max((size_t)c.per_chunk * 2 * M * sizeof(float2), (size_t)M * sizeof(double2));
+  if ((st = dalloc(p, &c.scratch, c.scratch_bytes)) != MADMAP_OK) return st;
+  double* G = nullptr;
+  if ((st = dalloc_t(p, &G, (size_t)p->n_filters * M)) != MADMAP_OK) return st;
+  c.G = G;   // set last: the setup is complete
+  return MADMAP_OK;
+}
+
+// grad[filter][tau] from p->bw_a and p->bw_r (corr_setup done).
+madmap_status corr_run(Plan* p, double* grad, cudaStream_t s) {
+  CorrPlan& c = p->corr;
+  MM_CUDA(cudaMemsetAsync(c.G, 0, sizeof(double) * (size_t)p->n_filters * c.M, s));
+  madmap_status st = corr_spectrum(p, s);
+  if (st != MADMAP_OK) return st;
+  SpecArgs a = {};
+  a.M = c.M;
+  a.logN1 = c.logN1;
+  a.logN2 = c.logN2;
+  a.n_lags = p->n_lags;
+  a.x = c.G;
+  a.tw = c.tw;
+  a.scratch = static_cast<double2*>(c.scratch);
+  a.reg_logN1 = c.reg.logN1;
+  a.grad = grad;
+  return run_spec<CORR>(a, p->n_filters, (int)std::min<size_t>(65535, c.scratch_bytes / ((size_t)c.M * sizeof(double2))), s);
+}
+
+}  // namespace mm

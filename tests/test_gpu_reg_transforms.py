@@ -55,3 +55,30 @@ def test_operator_matches_oracle(lg, runs):
     assert rel_rms(y, S.H(x.astype(np.float64))) < 2 * TOL   # two weights and a sum more per sample
     b = host(plan.rhs(cuda(p.d), precision="fp32"))[0]
     assert rel_rms(b, S.rhs(p.d[0])) < 2 * TOL
+
+
+@pytest.mark.parametrize("lg", [13, 14, 15, 16, 17, 18, 19])
+def test_lag_gradient_matches_direct_correlation(lg):
+    """The backward pass's lag correlation by windowed transforms, on intervals
+    shorter than a window, ending in its first sample, and of several windows
+    (their number odd, so that one window is alone), against direct sums.
+
+    A lag is an inner product of a = A lambda and a shifted r = d - A m, both
+    ways: a relative change of TOL in the norm of either (float32 inputs, one
+    float32 transform) moves it by at most 4 TOL |a| |r|."""
+    from oracle.adjoint import solve_backward
+    n_lags = 257
+    M = 1 << lg
+    exact = M - 2 * (n_lags - 1) if 14 <= lg <= 18 else (1 << 14) - 2 * (n_lags - 1)
+    p = tiny_T(seed=130 + lg, n=3 * exact + 1202, width=24, n_lags=n_lags, ivls=(1, 1200, exact + 1, 2 * exact))
+    S = system_for(p)
+    plan = make_plan(p, fft_len=M)
+    d = cuda(p.d[0])
+    m, _ = plan.solve(d, precision="fp64", rel_tol=1e-12, max_iter=1000)
+    g = np.random.default_rng(lg).standard_normal(tuple(m.shape))
+    _, gl, _ = plan.solve_backward(d, m, cuda(g), precision="fp64", rel_tol=1e-12, max_iter=1000)
+    d64 = p.d[0].astype(np.float64)
+    _, ogl, _ = solve_backward(S, d64, host(m), g)
+    lam, _ = S.pcg(g, rel_tol=1e-13, max_iter=2000)
+    scale = np.linalg.norm(S.unpoint(lam)) * np.linalg.norm(d64 - S.unpoint(host(m)))
+    assert np.abs(host(gl) - ogl).max() < 4 * TOL * scale, np.abs(host(gl) - ogl).max() / scale
