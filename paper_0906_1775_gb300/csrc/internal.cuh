@@ -85,8 +85,11 @@ struct __align__(8) df64 {
   __host__ __device__ constexpr df64(double v) : hi((float)v), lo((float)(v - (double)(float)v)) {}
   __host__ __device__ constexpr df64(float h, float l) : hi(h), lo(l) {}
 };
+// A complex double-float number: the real and imaginary parts' high words as
+// one register pair, their low words as another, so that packed float32
+// instructions do both parts' arithmetic (the operations below).
 struct __align__(16) cdf64 {
-  df64 x, y;
+  float2 h, l;   // (re, im)
 };
 __host__ __device__ inline double to_double(df64 a) { return (double)a.hi + (double)a.lo; }
 __device__ __forceinline__ df64 df_renorm(float s, float e) {
@@ -112,6 +115,48 @@ __device__ __forceinline__ df64 operator*(df64 a, df64 b) {
 __device__ __forceinline__ df64& operator+=(df64& a, df64 b) { return a = a + b; }
 __device__ __forceinline__ df64& operator-=(df64& a, df64 b) { return a = a - b; }
 __device__ __forceinline__ df64& operator*=(df64& a, df64 b) { return a = a * b; }
+
+// ---------------------------------------------------------------- packed float32
+// Two float32 operations in one instruction, each rounded as the scalar one.
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) {
+  unsigned long long r;
+  asm("sub.rn.f32x2 %0, %1, %2;"
+      : "=l"(r)
+      : "l"(reinterpret_cast<const unsigned long long&>(a)), "l"(reinterpret_cast<const unsigned long long&>(b)));
+  return reinterpret_cast<const float2&>(r);
+}
+__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
+
+// Complex double-float arithmetic, the df64 operations on both parts at once:
+// a complex sum is 11 packed instructions where two df64 sums were 22 (the
+// double-float operator on 97 tiles of 2^17: rows 145 -> 118, columns 188 ->
+// 165 and 214 -> 196 us per launch, one application 1031 -> 884 us; three row
+// CTAs per SM instead of two are 4 us of that).
+__device__ __forceinline__ cdf64 cdf_renorm(float2 s, float2 e) {
+  cdf64 r;
+  r.h = add2(s, e);
+  r.l = sub2(e, sub2(r.h, s));
+  return r;
+}
+__device__ __forceinline__ cdf64 cdf_sum(float2 ah, float2 bh, float2 lows) {
+  const float2 s = add2(ah, bh), bb = sub2(s, ah);
+  const float2 e = add2(sub2(ah, sub2(s, bb)), sub2(bh, bb));
+  return cdf_renorm(s, add2(e, lows));
+}
+// a b of the parts (a.x b.x, a.y b.y), not renormalised: heads in p, the rest in e
+__device__ __forceinline__ void cdf_mul_parts(const cdf64& a, float2 bh, float2 bl, float2& p, float2& e) {
+  p = __fmul2_rn(a.h, bh);
+  e = __ffma2_rn(a.h, bh, neg2(p));
+  e = __ffma2_rn(a.h, bl, e);
+  e = __ffma2_rn(a.l, bh, e);
+}
+// both parts times one real number
+__device__ __forceinline__ cdf64 cdf_scale(const cdf64& a, df64 b) {
+  float2 p, e;
+  cdf_mul_parts(a, make_float2(b.hi, b.hi), make_float2(b.lo, b.lo), p, e);
+  return cdf_renorm(p, e);
+}
 
 // ---------------------------------------------------------------- compressed pointing
 // Division of a detector sample index j >= 0 by the node step: a shift for a
@@ -572,6 +617,55 @@ __device__ __forceinline__ C csub(C a, C b) {
   return r;
 }
 
+// double-float: packed (see cdf64).  The products' tails join the sum's, so a
+// complex product renormalises once.
+__device__ __forceinline__ cdf64 cadd(const cdf64& a, const cdf64& b) { return cdf_sum(a.h, b.h, add2(a.l, b.l)); }
+__device__ __forceinline__ cdf64 csub(const cdf64& a, const cdf64& b) {
+  const float2 s = sub2(a.h, b.h), bb = sub2(s, a.h);
+  const float2 e = sub2(sub2(a.h, sub2(s, bb)), add2(b.h, bb));
+  return cdf_renorm(s, add2(e, sub2(a.l, b.l)));
+}
+__device__ __forceinline__ cdf64 cdf_times(const cdf64& a, const cdf64& b, float s) {  // s = 1: a b, s = -1: a conj(b)
+  float2 p, e, q, f;
+  cdf64 t;                      // (-a.y, a.x) for a b, (a.y, -a.x) for a conj(b)
+  t.h = make_float2(-s * a.h.y, s * a.h.x);
+  t.l = make_float2(-s * a.l.y, s * a.l.x);
+  cdf_mul_parts(a, make_float2(b.h.x, b.h.x), make_float2(b.l.x, b.l.x), p, e);
+  cdf_mul_parts(t, make_float2(b.h.y, b.h.y), make_float2(b.l.y, b.l.y), q, f);
+  return cdf_sum(p, q, add2(e, f));
+}
+__device__ __forceinline__ cdf64 cmul(const cdf64& a, const cdf64& b) { return cdf_times(a, b, 1.0f); }
+__device__ __forceinline__ cdf64 cmulc(const cdf64& a, const cdf64& b) { return cdf_times(a, b, -1.0f); }
+
+// parts of a complex number and its product with a real one
+template <typename C, typename R>
+__device__ __forceinline__ C make_c(R x, R y) {
+  C z;
+  z.x = x;
+  z.y = y;
+  return z;
+}
+template <>
+__device__ __forceinline__ cdf64 make_c<cdf64, df64>(df64 x, df64 y) {
+  cdf64 z;
+  z.h = make_float2(x.hi, y.hi);
+  z.l = make_float2(x.lo, y.lo);
+  return z;
+}
+__device__ __forceinline__ float c_re(float2 z) { return z.x; }
+__device__ __forceinline__ float c_im(float2 z) { return z.y; }
+__device__ __forceinline__ double c_re(double2 z) { return z.x; }
+__device__ __forceinline__ double c_im(double2 z) { return z.y; }
+__device__ __forceinline__ df64 c_re(const cdf64& z) { return df64(z.h.x, z.l.x); }
+__device__ __forceinline__ df64 c_im(const cdf64& z) { return df64(z.h.y, z.l.y); }
+__device__ __forceinline__ float2 c_scale(float2 z, float r) { return make_float2(z.x * r, z.y * r); }
+__device__ __forceinline__ double2 c_scale(double2 z, double r) { return make_double2(z.x * r, z.y * r); }
+__device__ __forceinline__ cdf64 c_scale(const cdf64& z, df64 r) { return cdf_scale(z, r); }
+template <typename C> struct RealOf;
+template <> struct RealOf<float2> { typedef float type; };
+template <> struct RealOf<double2> { typedef double type; };
+template <> struct RealOf<cdf64> { typedef df64 type; };
+
 // Shared-memory layout of the FFT buffers.  Rows sit `rs` elements apart and
 // element i of a row is stored at swz<SW>(i): bits 0-3 of i XORed with bits
 // 3-6 (SW = 0) or with bits 3-6 XOR bits 4-7 (SW = 1).  Both maps permute
@@ -599,6 +693,15 @@ constexpr int OP_THREADS = 256;
 
 // Multiplication by the constant w8^k = exp(-2 pi i k / 8), k = 0..3, or its
 // conjugate, written out so no general complex product is spent on it.
+template <int K, bool CONJ>
+__device__ __forceinline__ cdf64 mul_w8(const cdf64& v) {
+  if (K == 0) return v;
+  cdf64 t;                      // -i v (conj: i v)
+  t.h = CONJ ? make_float2(-v.h.y, v.h.x) : make_float2(v.h.y, -v.h.x);
+  t.l = CONJ ? make_float2(-v.l.y, v.l.x) : make_float2(v.l.y, -v.l.x);
+  if (K == 2) return t;
+  return cdf_scale(K == 1 ? cadd(v, t) : csub(t, v), df64(0.70710678118654752440));
+}
 template <int K, bool CONJ, typename C>
 __device__ __forceinline__ C mul_w8(C v) {
   typedef decltype(v.x) R;
@@ -847,7 +950,7 @@ __device__ __forceinline__ void reg_pass8(C (&v)[8], const C* tw, int logN, int 
 // transform leaves it).
 template <typename C, int R, int SW, typename HF>
 __device__ __forceinline__ void fused_middle(C* buf, int rows, int rs, int logN, int s, HF Hrow) {
-  typedef decltype(C().x) Real;
+  typedef typename RealOf<C>::type Real;
   const PassGeom G(logN, s, R);
   const int total = rows << G.gpr_log;
 #pragma unroll 4
@@ -868,10 +971,7 @@ __device__ __forceinline__ void fused_middle(C* buf, int rows, int rs, int logN,
     // filter product remains.
     small_dft<C, R, false>(v);
 #pragma unroll
-    for (int m = 0; m < (1 << R); ++m) {
-      v[m].x *= hv[m];
-      v[m].y *= hv[m];
-    }
+    for (int m = 0; m < (1 << R); ++m) v[m] = c_scale(v[m], hv[m]);
     small_dft<C, R, true>(v);
 #pragma unroll
     for (int m = 0; m < (1 << R); ++m) rp[swz<SW>(base + m * G.hR)] = v[m];

@@ -848,8 +848,7 @@ __global__ void __launch_bounds__(256, sizeof(Real) == 4 ? MM_MINB_F13 : MM_MINB
         gather_samples<Real, NS, IN, U>(a, L, nn, v);
 #pragma unroll
         for (int k = 0; k < U; ++k) {
-          gv[U * b + k].x = v[0][k];
-          gv[U * b + k].y = v[1][k];
+          gv[U * b + k] = make_c<C, Real>(v[0][k], v[1][k]);
         }
       }
       const int base = p0 + (G << (lgh - 1));
@@ -868,10 +867,7 @@ __global__ void __launch_bounds__(256, sizeof(Real) == 4 ? MM_MINB_F13 : MM_MINB
       for (int u = 0; u < U; ++u) {
         const int e = e0 + u * bd;
         if (e < total) {
-          C z;
-          z.x = v[0][u];
-          z.y = v[1][u];
-          buf[(e & (B1 - 1)) * rs + swz<SW>(e >> logB1)] = z;
+          buf[(e & (B1 - 1)) * rs + swz<SW>(e >> logB1)] = make_c<C, Real>(v[0][u], v[1][u]);
         }
       }
     }
@@ -920,7 +916,7 @@ __global__ void __launch_bounds__(256, sizeof(Real) == 4 ? MM_MINB_F13 : MM_MINB
 // ---------------------------------------------------------------- k_f2
 // LG1 > 0 fixes the row length N1 = 2^LG1 at compile time.
 template <typename Real, int LG1>
-__global__ void __launch_bounds__(256, sizeof(Real) == 4 ? 4 : 2) k_f2(OpArgs a) {
+__global__ void __launch_bounds__(256, sizeof(Real) == 4 ? 4 : 3) k_f2(OpArgs a) {
   typedef typename CxT<Real>::type C;
   constexpr int ELOG = elog<Real>();
   const int logN1 = LG1 ? LG1 : a.logN1;
@@ -1111,8 +1107,8 @@ __global__ void __launch_bounds__(256, sizeof(Real) == 4 ? MM_MINB_F13 : MM_MINB
 #pragma unroll
         for (int k = 0; k < U; ++k) {
           nn[k] = position(threadIdx.x + (2 * (U * b + k) + G) * bd);
-          val[0][k] = gv[U * b + k].x;
-          val[1][k] = gv[U * b + k].y;
+          val[0][k] = c_re(gv[U * b + k]);
+          val[1][k] = c_im(gv[U * b + k]);
         }
         scatter_samples<Real, NS, OUT, U, RUNB>(a, L, nn, val, hacc, hgrp);
       }
@@ -1125,11 +1121,10 @@ __global__ void __launch_bounds__(256, sizeof(Real) == 4 ? MM_MINB_F13 : MM_MINB
       for (int u = 0; u < U; ++u) {
         const int e = e0 + u * bd;
         nn[u] = position(e);
-        C z;
-        z.x = z.y = 0;
+        C z = make_c<C, Real>(Real(0), Real(0));
         if (e < total) z = buf[(e & (B1 - 1)) * rs + swz<SW>(e >> logB1)];
-        val[0][u] = z.x;
-        val[1][u] = z.y;
+        val[0][u] = c_re(z);
+        val[1][u] = c_im(z);
       }
       scatter_samples<Real, NS, OUT, U, RUNB>(a, L, nn, val, hacc, hgrp);
     }

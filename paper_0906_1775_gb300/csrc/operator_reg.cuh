@@ -55,21 +55,12 @@ __device__ __forceinline__ float2 mul_w32(float2 v, int k) {
   return make_float2(v.x * c + v.y * s, v.y * c - v.x * s);
 }
 
-// Complex sums, one packed instruction each (two float32 lanes of the register
-// pair, rounded as the scalar sums): the row kernel issues on 69% of its cycles
-// and half of its instructions were these (ring scan, 2^18: rows 46.7 -> 42.5,
-// inverse columns 113 -> 103 us per launch, one application 416 -> 387 us).
-__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 sub2(float2 a, float2 b) {
-  unsigned long long r;
-  asm("sub.rn.f32x2 %0, %1, %2;"
-      : "=l"(r)
-      : "l"(reinterpret_cast<const unsigned long long&>(a)), "l"(reinterpret_cast<const unsigned long long&>(b)));
-  return reinterpret_cast<const float2&>(r);
-}
-
 // 2^LG-point DFT (INV: inverse, unnormalised) of registers, natural order in,
 // bit-reversed order out: radix-2 decimation in frequency, constant twiddles.
+// Complex sums are one packed instruction each (add2, sub2): the row kernel
+// issued on 69% of its cycles and half of its instructions were these (ring
+// scan, 2^18: rows 46.7 -> 42.5, inverse columns 113 -> 103 us per launch, one
+// application 416 -> 387 us).
 template <int LG, bool INV>
 __device__ __forceinline__ void reg_dft(float2 (&v)[1 << LG]) {
 #pragma unroll

@@ -1376,8 +1376,9 @@ static madmap_status setup_windows(Plan* p, int M, long long tpc_req, cudaStream
       const double ang = 2.0 * M_PI * (double)j / (double)p->M;
       t64[j] = make_double2(cos(ang), -sin(ang));
       t32[j] = make_float2((float)t64[j].x, (float)t64[j].y);
-      tdf[j].x = df64(t64[j].x);
-      tdf[j].y = df64(t64[j].y);
+      const df64 c(t64[j].x), si(t64[j].y);
+      tdf[j].h = make_float2(c.hi, si.hi);
+      tdf[j].l = make_float2(c.lo, si.lo);
     }
     if ((st = walloc_t(p, &p->tw64, p->M)) != MADMAP_OK) return st;
     if (rl == 0 && (st = walloc_t(p, &p->tw32, p->M)) != MADMAP_OK) return st;
