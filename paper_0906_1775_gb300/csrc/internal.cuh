@@ -314,6 +314,17 @@ struct RegTables {
   const float4* four = nullptr;   // [N1][2]  w_n1 = exp(-2 pi i 16 n1 / M)
   const float2* four0 = nullptr;  // [16][N1] exp(-2 pi i n1 p / M)
 };
+// The float64-size types read every twiddle: complex entries in one array,
+// [16][16] exp(-2 pi i p j / 256); row_f [RA][RB] exp(-2 pi i p l / N1) and row_i
+// [RB][RA], the same transposed (N1 = RA RB as the row kernel splits it); row
+// [N1] exp(-2 pi i m / N1) for the shared-memory row kernel; four [256][N1]
+// exp(-2 pi i n1 k2 / M).
+constexpr int WIDE_ROW_F = 256;
+__host__ __device__ constexpr int wide_row_i(int logN1) { return WIDE_ROW_F + (1 << logN1); }
+__host__ __device__ constexpr int wide_row(int logN1) { return WIDE_ROW_F + (2 << logN1); }
+__host__ __device__ constexpr int wide_four(int logN1) { return WIDE_ROW_F + (3 << logN1); }
+// rows per exchange step of the row kernel (its RB = 2^lb lanes per row)
+__host__ __device__ constexpr int wide_lb(int logN1) { return logN1 >= 10 ? 5 : logN1 >= 8 ? 4 : 3; }
 constexpr int REG_N2 = 256;       // column length of the register transforms
 // log2(N1) of the register transforms of length M, or 0.
 inline int reg_log_n1(int M) { return (M >= (1 << 14) && M <= (1 << 18)) ? __builtin_ctz((unsigned)M) - 8 : 0; }
@@ -363,10 +374,13 @@ struct Plan {
   float* P32 = nullptr;            // [n_obs][8] (IQU) or [n_obs] (T)
   Tile* tiles = nullptr;           // [n_tiles]
   double* H64 = nullptr;           // [n_filters][M] permuted spectra / M
-  float* H32 = nullptr;            // as H64, or [k2][k1] natural order for register transforms
+  float* H32 = nullptr;            // (register transforms: [k2][k1] natural order; the wide types' rows of
+                                   // more than 256 points bit-reversed in k1)
   double2* tw64 = nullptr;         // [M] exp(-2 pi i j / M)
   float2* tw32 = nullptr;          // (NULL with register transforms)
-  RegTables reg;                   // float32 register transforms
+  RegTables reg;                   // register transforms: float32 tables,
+  double2* wide64 = nullptr;       // float64 ones
+  cdf64* wide_df = nullptr;        // and double-float ones (see wide_four)
   df64* Hdf = nullptr;             // [n_filters][M] H64 as double-float pairs
   cdf64* twdf = nullptr;           // [M] tw64 as double-float pairs
   float4* csdf = nullptr;          // [n_t] cs64 as double-float pairs (IQU)
@@ -562,6 +576,8 @@ madmap_status ensure_wtod(Plan* p, int n_rhs);
 
 // Spectra of p->lags into H64, H32, Hdf on the device (spectra.cu); waits for s.
 madmap_status build_spectra(Plan* p, cudaStream_t s);
+// The wide register tables of p->M from tw64 and twdf (spectra.cu).
+madmap_status fill_wide_tables(Plan* p, cudaStream_t s);
 
 // Backward pass: lag correlation of p->bw_a by transforms where corr_by_fft;
 // corr_spectrum (operator_f32.cu) sums the windows' cross spectra into corr.G.

@@ -27,7 +27,7 @@ madmap_status corr_spectrum(Plan* p, cudaStream_t s) {
   for (int t0 = 0; t0 < c.n_pairs; t0 += c.per_chunk) {
     const int n = std::min(c.per_chunk, c.n_pairs - t0);
     a.tile0 = 2 * t0;
-    k_c1<1, IN_TODF><<<dim3((1 << a.reg_logN1) / REG_COLS, 2 * n), 256, 0, s>>>(a);
+    k_c1<float, 1, IN_TODF, 16><<<dim3((1 << a.reg_logN1) / 16, 2 * n), 256, 0, s>>>(a);
     switch (a.reg_logN1) {
       case 6: k_xcorr<3, 3><<<dim3(256 / RowGeom<3, 3>::ROWS, n), 128, 0, s>>>(a, c.G); break;
       case 7: k_xcorr<4, 3><<<dim3(256 / RowGeom<4, 3>::ROWS, n), 128, 0, s>>>(a, c.G); break;

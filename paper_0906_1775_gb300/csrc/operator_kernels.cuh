@@ -109,6 +109,7 @@ struct OpArgs {
   int reg_logN1;
   const float4 *reg_col, *reg_row, *reg_four;
   const float2* reg_four0;
+  const void* reg_wide;  // the float64-size types' (WideTables)
   int n_rep;          // > 1: map outputs go to replica (blockIdx.x + blockIdx.y) % n_rep, rep_stride apart
   int runs;           // scatter runs of consecutive samples that hit one pixel with one atomic (run_*)
   long long rep_stride;
@@ -1140,7 +1141,30 @@ __global__ void __launch_bounds__(256, sizeof(Real) == 4 ? MM_MINB_F13 : MM_MINB
 }
 
 
-#include "operator_reg.cuh"  // k_c1, k_c2, k_c3 (float32)
+template <typename Real>
+inline int elems_per_cta() {
+  return 1 << elog<Real>();
+}
+
+typedef void (*OpKernel)(OpArgs);
+
+// Raise a kernel's dynamic shared-memory limit when a plan needs more than it
+// was last given (once per kernel instance and size; host-side bookkeeping).
+cudaError_t set_smem(OpKernel kernel, size_t bytes) {
+  static std::mutex mu;
+  static std::vector<std::pair<const void*, size_t>> done;
+  std::lock_guard<std::mutex> lk(mu);
+  for (auto& d : done)
+    if (d.first == (const void*)kernel) {
+      if (d.second >= bytes) return cudaSuccess;
+      d.second = bytes;
+      return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    }
+  done.push_back({(const void*)kernel, bytes});
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+
+#include "operator_reg.cuh"  // k_c1, k_c2, k_c3
 
 // ---------------------------------------------------------------- k_diag
 // White noise (one filter lag, e.g. destriping runs, Section 6 item 3): N^-1
@@ -1265,11 +1289,6 @@ __global__ void k_rep_reduce(Out* rep, int n_rep, long long stride, Out* out, lo
 }
 
 template <typename Real>
-inline int elems_per_cta() {
-  return 1 << elog<Real>();
-}
-
-template <typename Real>
 void geometry(const Plan* p, int& B1, int& B2) {
   const int E = elems_per_cta<Real>();
   B1 = E / p->N2;
@@ -1296,24 +1315,6 @@ size_t smem_f2(const Plan* p) {
          sizeof(typename CxT<Real>::type);
 }
 
-typedef void (*OpKernel)(OpArgs);
-
-// Raise a kernel's dynamic shared-memory limit when a plan needs more than it
-// was last given (once per kernel instance and size; host-side bookkeeping).
-cudaError_t set_smem(OpKernel kernel, size_t bytes) {
-  static std::mutex mu;
-  static std::vector<std::pair<const void*, size_t>> done;
-  std::lock_guard<std::mutex> lk(mu);
-  for (auto& d : done)
-    if (d.first == (const void*)kernel) {
-      if (d.second >= bytes) return cudaSuccess;
-      d.second = bytes;
-      return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    }
-  done.push_back({(const void*)kernel, bytes});
-  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
 // The three operator kernels for a plan: instances with compile-time FFT
 // geometry for the common sizes, the generic instances otherwise.
 struct OpKernels {
@@ -1323,47 +1324,37 @@ struct OpKernels {
 template <typename Real, int NS, int IN, int OUT>
 OpKernels pick_kernels(const Plan* p) {
   OpKernels k;
-  // the T on-the-fly and extended-pointing modes keep only the generic column
-  // kernels (fewer instances to compile)
+  // Lengths 2^14 .. 2^18 run in operator_reg.cuh (except in the allocation-free
+  // weighting's float64, a timestream in and out).  The others' columns have 128
+  // points (2^13), 1024 (2^19, 2^20), 512 (2^19 with fft_split), or few enough
+  // for the generic instance, which also serves the T on-the-fly and
+  // extended-pointing modes (fewer instances to compile).
   constexpr bool generic_only = NS == NS_OTF_T || extended(NS);
-  if constexpr (generic_only) {
-    k.f1 = k_f1<Real, NS, IN, 0>;
-    k.f3 = k_f3<Real, NS, OUT, 0>;
-  } else if constexpr (std::is_same<Real, float>::value) {
-    // lengths 2^14 .. 2^18 run in operator_reg.cuh: the others' columns have
-    // 128 (2^13), 512 (2^19 with fft_split) or 1024 points, or few enough for
-    // the generic instance
+  constexpr bool every = std::is_same<Real, double>::value && NS == 1 && IN == IN_TODR;
+  k.f1 = k_f1<Real, NS, IN, 0>;
+  k.f3 = k_f3<Real, NS, OUT, 0>;
+  if constexpr (!generic_only) {
     switch (p->logN2) {
       case 7: k.f1 = k_f1<Real, NS, IN, 7>; k.f3 = k_f3<Real, NS, OUT, 7>; break;
       case 9: k.f1 = k_f1<Real, NS, IN, 9>; k.f3 = k_f3<Real, NS, OUT, 9>; break;
       case 10: k.f1 = k_f1<Real, NS, IN, 10>; k.f3 = k_f3<Real, NS, OUT, 10>; break;
-      default: k.f1 = k_f1<Real, NS, IN, 0>; k.f3 = k_f3<Real, NS, OUT, 0>; break;
-    }
-  } else {
-    switch (p->logN2) {
-      case 7: k.f1 = k_f1<Real, NS, IN, 7>; k.f3 = k_f3<Real, NS, OUT, 7>; break;
-      case 8: k.f1 = k_f1<Real, NS, IN, 8>; k.f3 = k_f3<Real, NS, OUT, 8>; break;
-      case 9: k.f1 = k_f1<Real, NS, IN, 9>; k.f3 = k_f3<Real, NS, OUT, 9>; break;
-      case 10: k.f1 = k_f1<Real, NS, IN, 10>; k.f3 = k_f3<Real, NS, OUT, 10>; break;
-      default: k.f1 = k_f1<Real, NS, IN, 0>; k.f3 = k_f3<Real, NS, OUT, 0>; break;
     }
   }
-  if constexpr (std::is_same<Real, float>::value) {
-    switch (p->logN1) {
-      case 6: k.f2 = k_f2<Real, 6>; break;
-      case 9: k.f2 = k_f2<Real, 9>; break;
-      case 10: k.f2 = k_f2<Real, 10>; break;
-      default: k.f2 = k_f2<Real, 0>; break;
+  if constexpr (every) {
+    if (p->logN2 == 8) {
+      k.f1 = k_f1<Real, NS, IN, 8>;
+      k.f3 = k_f3<Real, NS, OUT, 8>;
     }
-  } else {
-    switch (p->logN1) {
-      case 6: k.f2 = k_f2<Real, 6>; break;
-      case 7: k.f2 = k_f2<Real, 7>; break;
-      case 8: k.f2 = k_f2<Real, 8>; break;
-      case 9: k.f2 = k_f2<Real, 9>; break;
-      case 10: k.f2 = k_f2<Real, 10>; break;
-      default: k.f2 = k_f2<Real, 0>; break;
-    }
+  }
+  k.f2 = k_f2<Real, 0>;
+  switch (p->logN1) {
+    case 6: k.f2 = k_f2<Real, 6>; break;
+    case 9: k.f2 = k_f2<Real, 9>; break;
+    case 10: k.f2 = k_f2<Real, 10>; break;
+  }
+  if constexpr (std::is_same<Real, double>::value) {
+    if (p->logN1 == 7) k.f2 = k_f2<Real, 7>;
+    if (p->logN1 == 8) k.f2 = k_f2<Real, 8>;
   }
   return k;
 }
@@ -1522,8 +1513,7 @@ madmap_status launch_all(Plan* p, const void* in, void* out, long long in_stride
   a.runs = p->runs;
   a.tiles = ts ? ts->tiles : p->tiles;
   const int n_tiles = ts ? ts->n_tiles : p->n_tiles;
-  constexpr bool F32 = std::is_same<Real, float>::value;
-  const bool reg = F32 && p->reg.logN1 > 0;   // register transforms (static shared memory)
+  const bool reg = p->reg.logN1 > 0;   // register transforms
   const size_t sm13 = smem_f13<Real>(p), sm2 = smem_f2<Real>(p);
   const OpKernels K = pick_kernels<Real, NS, IN, OUT>(p);
   a.reg_logN1 = p->reg.logN1;
@@ -1531,11 +1521,18 @@ madmap_status launch_all(Plan* p, const void* in, void* out, long long in_stride
   a.reg_row = p->reg.row;
   a.reg_four = p->reg.four;
   a.reg_four0 = p->reg.four0;
+  a.reg_wide = DF ? (const void*)p->wide_df : (const void*)p->wide64;
   // n_rhs == 0 only sets the kernels' attributes, so it can precede a capture
   if (!reg) {
     MM_CUDA(set_smem(K.f1, sm13));
     MM_CUDA(set_smem(K.f3, sm13));
     MM_CUDA(set_smem(K.f2, sm2));
+  } else if (sizeof(Real) == 8 && p->reg.logN1 >= 9) {
+    OpKernel f2;
+    int b2;
+    size_t sm;
+    const madmap_status st = wide_rows<Real>(p->reg.logN1, f2, b2, sm);
+    if (st != MADMAP_OK) return st;
   }
   if (p->diag && !ts) {
     // white noise: one diagonal pass per right-hand side (launch events as
@@ -1612,11 +1609,10 @@ madmap_status launch_all(Plan* p, const void* in, void* out, long long in_stride
         const cudaStream_t cs = pipe ? p->op_stream[chunk & 1] : s;
         a.scratch = scratch + (pipe ? (size_t)(chunk & 1) * slot_bytes : 0);
         ++chunk;
-        if constexpr (F32) {
-          if (reg) {
-            launch_reg<NS, IN, OUT>(a, nt, cs, ev, &ei);
-            continue;
-          }
+        if (reg) {
+          const madmap_status st = launch_reg<Real, NS, IN, OUT>(a, nt, cs, ev, &ei);
+          if (st != MADMAP_OK) return st;
+          continue;
         }
         dim3 g13(p->N1 / a.B1, nt), g2(p->N2 / a.B2, nt);
         if (ev) cudaEventRecord(ev[ei++], s);

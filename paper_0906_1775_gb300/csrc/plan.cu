@@ -81,6 +81,8 @@ static void free_windows(Plan* p) {
   p->tw64 = nullptr;
   p->tw32 = nullptr;
   p->reg = RegTables();
+  p->wide64 = nullptr;
+  p->wide_df = nullptr;
   p->twdf = nullptr;
   p->scratch = nullptr;
 }
@@ -1386,6 +1388,12 @@ static madmap_status setup_windows(Plan* p, int M, long long tpc_req, cudaStream
     MM_CUDA(cudaMemcpy(p->tw64, t64.data(), sizeof(double2) * p->M, cudaMemcpyHostToDevice));
     if (rl == 0) MM_CUDA(cudaMemcpy(p->tw32, t32.data(), sizeof(float2) * p->M, cudaMemcpyHostToDevice));
     MM_CUDA(cudaMemcpy(p->twdf, tdf.data(), sizeof(cdf64) * p->M, cudaMemcpyHostToDevice));
+    if (rl > 0) {
+      const size_t n = (size_t)wide_four(rl) + p->M;
+      if ((st = walloc_t(p, &p->wide64, n)) != MADMAP_OK) return st;
+      if ((st = walloc_t(p, &p->wide_df, n)) != MADMAP_OK) return st;
+      if ((st = fill_wide_tables(p, s)) != MADMAP_OK) return st;
+    }
   }
   {
     const int n_chunks = p->n_tiles ? (p->n_tiles + p->tiles_per_chunk - 1) / p->tiles_per_chunk : 0;

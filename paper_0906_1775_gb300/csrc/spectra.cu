@@ -100,12 +100,15 @@ __global__ void __launch_bounds__(OP_THREADS) k_spec_rows(SpecArgs a) {
       // a NaN orders above +inf as positive, so it is mapped below every value
       const unsigned long long b = v == v ? order_bits(v) : 0ull;
       mn = b < mn ? b : mn;
-      const long long o = (long long)f * a.M + ((long long)pos2 << a.logN1) + pos1;
+      long long o = (long long)f * a.M + ((long long)pos2 << a.logN1) + pos1, r = o;
+      if (a.reg_logN1 > 0) {
+        const int k1 = k >> 8;
+        o = r = (long long)f * a.M + ((long long)(k & (REG_N2 - 1)) << a.reg_logN1);
+        r += k1;
+        o += a.reg_logN1 > 8 ? brev_n(k1, a.reg_logN1) : k1;
+      }
       a.H64[o] = v;
       a.Hdf[o] = df64((float)v, (float)(v - (double)(float)v));
-      const long long r = a.reg_logN1 > 0
-                              ? (long long)f * a.M + ((long long)(k & (REG_N2 - 1)) << a.reg_logN1) + (k >> 8)
-                              : o;
       a.H32[r] = (float)v;
     } else if (k < a.n_lags) {
       // c(tau) + c(-tau) = sum_k 2 G cos / M; tau = 0 counts once
@@ -127,6 +130,30 @@ __global__ void k_fill_twiddles(double2* tw, int M) {
     double s, c;
     sincospi(2.0 * (double)j / (double)M, &s, &c);
     tw[j] = make_double2(c, -s);
+  }
+}
+
+// WideTables of length M = 256 N1 from the table of M-th roots.
+template <typename C>
+__global__ void k_wide_tables(const C* tw, C* out, int logN1) {
+  const int N1 = 1 << logN1, M = N1 << 8, lb = wide_lb(logN1), la = logN1 - lb, n = wide_four(logN1) + M;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    int m;
+    if (i < WIDE_ROW_F) {
+      m = (i >> 4) * (i & 15) * N1;
+    } else if (i < wide_row_i(logN1)) {
+      const int e = i - WIDE_ROW_F;
+      m = (e >> lb) * (e & ((1 << lb) - 1)) * REG_N2;
+    } else if (i < wide_row(logN1)) {
+      const int e = i - wide_row_i(logN1);
+      m = (e >> la) * (e & ((1 << la) - 1)) * REG_N2;
+    } else if (i < wide_four(logN1)) {
+      m = (i - wide_row(logN1)) * REG_N2;
+    } else {
+      const int e = i - wide_four(logN1);
+      m = (e >> logN1) * (e & (N1 - 1));
+    }
+    out[i] = tw[m & (M - 1)];
   }
 }
 
@@ -163,6 +190,14 @@ madmap_status run_spec(SpecArgs a, int n_f, int batch, cudaStream_t s) {
 }
 
 }  // namespace
+
+madmap_status fill_wide_tables(Plan* p, cudaStream_t s) {
+  const int rl = p->reg.logN1, grid = (wide_four(rl) + p->M + 255) / 256;
+  k_wide_tables<double2><<<grid, 256, 0, s>>>(p->tw64, p->wide64, rl);
+  k_wide_tables<cdf64><<<grid, 256, 0, s>>>(p->twdf, p->wide_df, rl);
+  MM_CUDA(cudaGetLastError());
+  return MADMAP_OK;
+}
 
 // The spectra of all filters (p->lags) into p->H64, p->H32 and p->Hdf, using
 // p->tw64 and p->scratch; waits for the stream and fails when a symbol is not
