@@ -27,6 +27,7 @@
 // right-hand side, each stops on its own, and the operator takes a tile set
 // whose lanes pair right-hand sides of one window (so they share one FFT and
 // one pass over the pointing) and skips tiles whose right-hand sides are done.
+#include <cooperative_groups.h>
 #include <math.h>
 #include <stdlib.h>
 
@@ -487,6 +488,170 @@ __global__ void __launch_bounds__(NT) k_cg_direction(const Real* x, const Real* 
   }
 }
 
+// One whole iteration after the operator for maps of at most CG_STEP_ROWS rows:
+// k_cg_alpha, k_cg_update and k_cg_direction in one cluster of 8 CTAs, the
+// iteration's vectors in registers between the sums and the sums through
+// distributed shared memory (every CTA adds the eight partials in rank order).
+// Three launches of 16 CTAs on a 4096-row map cost 22 us of an 88 us float64
+// iteration, almost all of it launch and last-block latency; this one takes 10 us
+// (float64 solve of that map 1.52 -> 1.41 ms).  An SM's float64 pipe takes a
+// warp's instruction in some 16 cycles, so divisions and roots are left to one
+// thread (every thread computing them: 17.7 us), and 4 rows a thread keep the
+// warps that reduce few.  Larger maps keep the three kernels: 8 SMs would then
+// move the vectors slower than 152.
+constexpr int CG_CTAS = 8, CG_ROWS = 4;
+constexpr int CG_THREADS_S = 128, CG_THREADS_L = 512;
+constexpr int CG_STEP_ROWS = CG_CTAS * CG_THREADS_L * CG_ROWS;
+
+// The cluster's sum of v in thread 0 of every CTA (part: this CTA's list of the
+// CTAs' sums, warp: its warps').
+template <int K, int THREADS>
+__device__ __forceinline__ void cluster_sums(double (&v)[K], double (*part)[K], double (*warp)[K]) {
+  cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+#pragma unroll
+  for (int k = 0; k < K; ++k)
+    for (int off = 16; off > 0; off >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], off);
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  if (lane == 0)
+#pragma unroll
+    for (int k = 0; k < K; ++k) warp[wid][k] = v[k];
+  __syncthreads();
+  if (threadIdx.x < CG_CTAS) {   // thread c: this CTA's sum into CTA c's list
+    double (*dst)[K] = cl.map_shared_rank(part, threadIdx.x);
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      double s = 0.0;
+#pragma unroll
+      for (int w = 0; w < THREADS / 32; ++w) s += warp[w][k];
+      dst[cl.block_rank()][k] = s;
+    }
+  }
+  cl.sync();
+  if (threadIdx.x == 0) {
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      v[k] = 0.0;
+#pragma unroll
+      for (int c = 0; c < CG_CTAS; ++c) v[k] += part[c][k];
+    }
+  }
+}
+
+template <typename Real, int NS, int THREADS>
+__global__ void __cluster_dims__(CG_CTAS, 1, 1) __launch_bounds__(THREADS)
+    k_cg_step(Real* x, Real* r, Real* z, Real* p, Real* q, Real* xb, long long nvec, int n_obs, const double* P64,
+              const float* P32, const unsigned char* f64, CgState* st, double* hist) {
+  __shared__ double part1[CG_CTAS][1], part2[CG_CTAS][2];
+  __shared__ double warp1[THREADS / 32][1], warp2[THREADS / 32][2];
+  __shared__ double sc[2];   // alpha, then beta
+  __shared__ int flag[2];    // p.q > 0; then bit 0: better, bit 1: done
+  st += blockIdx.y;
+  if (st->halt) return;   // the whole cluster: the state changes after its first sync only
+  cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+  const long long o = blockIdx.y * nvec;
+  x += o; r += o; z += o; p += o; q += o; xb += o;
+  V3<Real, NS> pv[CG_ROWS], qv[CG_ROWS], xv[CG_ROWS], rv[CG_ROWS], zv[CG_ROWS];
+  double dot[1] = {0.0};
+  const int i0 = blockIdx.x * THREADS + threadIdx.x;
+#pragma unroll
+  for (int u = 0; u < CG_ROWS; ++u) {
+    const int i = i0 + u * CG_CTAS * THREADS;
+    if (i < n_obs) {
+      pv[u] = ldv<Real, NS>(p, i);
+      qv[u] = ldv<Real, NS>(q, i);
+      xv[u] = ldv<Real, NS>(x, i);
+      rv[u] = ldv<Real, NS>(r, i);
+    }
+  }
+  const CgState S = *st;
+  cl.sync();   // no CTA may write another's shared memory before that one runs
+#pragma unroll
+  for (int u = 0; u < CG_ROWS; ++u)
+    if (i0 + u * CG_CTAS * THREADS < n_obs) dot[0] += dotv(pv[u], qv[u]);
+  cluster_sums<1, THREADS>(dot, part1, warp1);
+  if (threadIdx.x == 0) {
+    const bool pd = dot[0] > 0.0 && isfinite(dot[0]);
+    flag[0] = pd;
+    sc[0] = pd ? S.rz / dot[0] : 0.0;
+    if (blockIdx.x == 0) {
+      if (pd) {
+        st->alpha = sc[0];
+      } else {
+        st->status = (int)MADMAP_ERR_NOT_PD;
+        st->done = 1;
+        st->halt = 1;
+      }
+    }
+  }
+  __syncthreads();
+  if (!flag[0]) return;   // the whole cluster
+  const Real alpha = (Real)sc[0];
+  double s[2] = {0.0, 0.0};
+#pragma unroll
+  for (int u = 0; u < CG_ROWS; ++u) {
+    const int i = i0 + u * CG_CTAS * THREADS;
+    if (i < n_obs) {
+      xv[u].a += alpha * pv[u].a;
+      rv[u].a -= alpha * qv[u].a;
+      if (NS == 3) {
+        xv[u].b += alpha * pv[u].b;
+        xv[u].c += alpha * pv[u].c;
+        rv[u].b -= alpha * qv[u].b;
+        rv[u].c -= alpha * qv[u].c;
+      }
+      zv[u] = precond<Real, NS>(rv[u], i, P64, P32, f64);
+      stv<Real, NS>(x, i, xv[u]);
+      stv<Real, NS>(r, i, rv[u]);
+      stv<Real, NS>(z, i, zv[u]);
+      s[0] += dotv(rv[u], zv[u]);
+      s[1] += dotv(rv[u], rv[u]);
+    }
+  }
+  cluster_sums<2, THREADS>(s, part2, warp2);
+  if (threadIdx.x == 0) {
+    const int k = S.k + 1;
+    const double res = sqrt(s[1]) / S.bnorm, beta = s[0] / S.rz;
+    const bool better = res < S.best_res;
+    const bool done = res <= S.tol || k >= S.max_iter || !isfinite(res);
+    sc[1] = beta;
+    flag[1] = (better ? 1 : 0) | (done ? 2 : 0);
+    if (blockIdx.x == 0) {
+      st->beta = beta;
+      st->rz = s[0];
+      st->k = k;
+      st->dir_k = k;
+      st->res = res;
+      if (hist && k < HIST_CAP) hist[(long long)blockIdx.y * HIST_CAP + k] = res;
+      if (better) {
+        st->best_res = res;
+        st->best_k = k;
+      }
+      if (done) st->done = 1;
+      st->halt = done || k >= S.pause_k;
+    }
+  }
+  __syncthreads();
+  const bool better = flag[1] & 1, more = !(flag[1] & 2);
+  const Real beta = (Real)sc[1];
+#pragma unroll
+  for (int u = 0; u < CG_ROWS; ++u) {
+    const int i = i0 + u * CG_CTAS * THREADS;
+    if (i < n_obs) {
+      if (better) stv<Real, NS>(xb, i, xv[u]);
+      if (more) {
+        pv[u].a = zv[u].a + beta * pv[u].a;
+        if (NS == 3) {
+          pv[u].b = zv[u].b + beta * pv[u].b;
+          pv[u].c = zv[u].c + beta * pv[u].c;
+        }
+        stv<Real, NS>(p, i, pv[u]);
+        const V3<Real, NS> zero = {0, 0, 0};
+        stv<Real, NS>(q, i, zero);
+      }
+    }
+  }
+}
+
 // Residual replacement: the float32 PCG continues across a refinement step
 // (the residual replacement of van der Vorst and Ye, 2000; the "reliable
 // updates" of Clark et al., 2010).  The recursive residual is replaced by
@@ -687,6 +852,17 @@ static void enqueue_iteration(Plan* p, SolveBuffers* sb, const Batch& B, cudaStr
   // sharded plans: q = sum over the ranks of their shares of H p
   if (*st == MADMAP_OK)
     *st = reduce_across(p, q, nv * B.n_rhs, sizeof(Real) == 8 ? MADMAP_REDUCE_F64 : MADMAP_REDUCE_F32, s);
+  if (n <= CG_STEP_ROWS) {
+    count_launches(1);
+    const dim3 gs(CG_CTAS, B.n_rhs);
+    if (n <= CG_CTAS * CG_THREADS_S * CG_ROWS)
+      k_cg_step<Real, NS, CG_THREADS_S><<<gs, CG_THREADS_S, 0, s>>>(x, r, z, pp, q, xb, nv, n, p->P64, p->P32,
+                                                                    p->fp64flag, sb->st, sb->hist);
+    else
+      k_cg_step<Real, NS, CG_THREADS_L><<<gs, CG_THREADS_L, 0, s>>>(x, r, z, pp, q, xb, nv, n, p->P64, p->P32,
+                                                                    p->fp64flag, sb->st, sb->hist);
+    return;
+  }
   count_launches(3);
   k_cg_alpha<Real, NS><<<g, NT, 0, s>>>(pp, q, nv, n, sb->st, sb->partials);
   k_cg_update<Real, NS><<<g, NT, 0, s>>>(x, r, z, pp, q, nv, n, p->P64, p->P32, p->fp64flag, sb->st, sb->partials,
