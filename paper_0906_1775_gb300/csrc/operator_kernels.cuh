@@ -1238,7 +1238,86 @@ __global__ void __launch_bounds__(256) k_diag(OpArgs a, const DiagItem* __restri
   const LaneView<Real> L = lane_view<Real, IN, OUT>(a, g);
   const Real w0 = Real(f0[it.filter]);
   const int len = (int)(it.hi - it.lo);
-  if constexpr (!HWP) {
+  if constexpr (!HWP && gathers(IN) && OUT == OUT_MAP && !(std::is_same<Real, df64>::value && polarised(NS))) {
+    // map to map: a sample's pointing is read once for both sides, U samples in
+    // flight; whole-block rounds, so that every warp stays converged for the
+    // extra columns' sums, which a baseline's samples add up in registers.
+    // Bound by requests for scattered map lines (L1 tags and the crossbar near
+    // 70% of their rates): destriping pass of 4 x 2^22 samples, 512 x 512 map,
+    // 155 -> 110 us (201 MB of pointing and columns: 1.3 -> 1.8 TB/s) against
+    // reading the pointing twice and matching columns lane by lane.
+    typedef typename OutT<Real>::type Out;
+    constexpr int U = 2, EXT = map_ns(NS) == 3 ? 4 : 1;
+    Out* y = static_cast<Out*>(L.out);
+    // extra column of the warp's samples so far (the same in every lane) and
+    // this lane's share of its sum
+    int col = -1;
+    Out share = Out(0);
+    auto flush = [&]() {
+      if (col >= 0) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) share += __shfl_xor_sync(0xffffffffu, share, o);
+        if ((threadIdx.x & 31) == 0) atomicAdd(y + (long long)col * EXT, share);
+      }
+      share = Out(0);
+    };
+    for (int n0 = 0; n0 < len; n0 += U * 256) {
+      int pp[U], qq[U];
+      Real c[U], sn[U], v[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int n = n0 + u * 256 + (int)threadIdx.x;
+        load_pointing<Real, NS>(a, L, n, n < len, pp[u], c[u], sn[u]);
+        qq[u] = -1;
+        if constexpr (NS == NS_MR || extended(NS)) {
+          const int* qp = NS == NS_MR ? L.pq : L.pe;
+          if (n < len && qp) qq[u] = __ldg(qp + n);
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int n = n0 + u * 256 + (int)threadIdx.x;
+        if (polarised(NS) && !on_the_fly(NS)) finish_angle<Real>(c[u], sn[u]);
+        const Real* x = static_cast<const Real*>(L.in);
+        v[u] = Real(0);
+        if (pp[u] >= 0) {
+          if constexpr (NS == NS_MR) v[u] = gather_mr<Real>(x, pp[u], qq[u], c[u], sn[u]);
+          else v[u] = gather<Real, map_ns(NS)>(x, pp[u], c[u], sn[u]);
+          if constexpr (extended(NS))
+            if (qq[u] >= 0) v[u] += x[(long long)qq[u] * EXT];
+        }
+        if constexpr (IN == IN_RESX)
+          if (n < len) v[u] = Real(__ldg(L.in2 + n)) - v[u];
+        v[u] = v[u] * w0;
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        if (pp[u] >= 0) {
+          if constexpr (NS == NS_MR) scatter_mr<Real>(y, pp[u], qq[u], v[u], c[u], sn[u]);
+          else scatter<Real, map_ns(NS)>(y, pp[u], v[u], c[u], sn[u]);
+        }
+        if constexpr (extended(NS)) {
+          const bool in = n0 + u * 256 + (int)threadIdx.x < len;
+          const bool adds = pp[u] >= 0 && qq[u] >= 0;
+          const unsigned m = __ballot_sync(0xffffffffu, in);
+          if (m) {   // the same in every lane
+            const int e0 = __shfl_sync(0xffffffffu, qq[u], __ffs(m) - 1);
+            if (__all_sync(0xffffffffu, !in || qq[u] == e0)) {
+              if (e0 != col) {
+                flush();
+                col = e0;
+              }
+              if (adds) share += (Out)to_out(v[u]);
+            } else if (adds) {   // a boundary inside the warp
+              atomic_add_warp(y, (long long)qq[u] * EXT, (Out)to_out(v[u]));
+            }
+            __syncwarp();
+          }
+        }
+      }
+    }
+    if constexpr (extended(NS)) flush();
+  } else if constexpr (!HWP) {
     for (int n = threadIdx.x; n < len; n += blockDim.x) {
       Real v;
       if (IN == IN_MAPX) v = sample_gather<Real, NS>(a, L, n);
