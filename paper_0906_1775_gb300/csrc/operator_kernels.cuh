@@ -1141,6 +1141,90 @@ __global__ void __launch_bounds__(256, sizeof(Real) == 4 ? MM_MINB_F13 : MM_MINB
 }
 
 
+// Lanes of a run sum (run_sum): a run of samples in one pixel adds once per
+// aligned group of this many.  Four takes two shuffle steps of each of the three
+// sums where a warp row of 16 samples takes four, for one atomic in two samples
+// instead of one in three on the ring scan (0.65 repeats); the shuffles were a
+// third of k_c3's L1 wavefronts (16, 8, 4 lanes: 103.5, 97.9, 97.6 us per launch,
+// 387, 377, 373 us per application).
+constexpr int REG_RUN = 4;
+
+// ---------------------------------------------------------------- k_one
+// A whole tile in one CTA, for windows that fit its shared memory: gather, FFT,
+// filter, inverse FFT and outputs in one launch, with no scratch.  (A transform
+// of M = N1 N2 points in one row leaves the bit-reversed order that the
+// spectrum's [N2 position][N1 position] is in.)  Short problems wait for launches
+// and each CTA's first loads, long ones for the two trips through scratch:
+// weighting of 5000 samples (M = 1024) 21.9 -> 18.5 us a call, of 10^6 samples
+// (M = 2048) 32.3 -> 24.9 us, IQU operator of 4 x 2^20 samples (M = 2048) 73.6 ->
+// 63.9 us.  Up to 100 KB, so two CTAs share an SM: at 128 KB (float32 M = 8192)
+// one IQU application takes 80 us where the three kernels take 71.
+template <typename Real, int NS, int IN, int OUT>
+__global__ void __launch_bounds__(OP_THREADS, 2) k_one(OpArgs a) {
+  typedef typename CxT<Real>::type C;
+  typedef typename OutT<Real>::type Out;
+  const Tile* T = a.tiles + a.tile0 + blockIdx.x;
+  if (skip_tile(a, T)) return;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  constexpr int SW = 1;
+  const int logM = a.logN1 + a.logN2;
+  C* buf = reinterpret_cast<C*>(smem_raw);
+  const int rs = lay_rs(sizeof(C), logM, false);
+  C* tw = buf + rs;
+  build_pass_twiddles(tw, logM, static_cast<const C*>(a.tw), 1);
+  constexpr bool HWP = extended(NS) && OUT == OUT_MAP;
+  __shared__ Out hacc[HWP ? 64 : 1];
+  __shared__ int hgrp[2];
+  if (HWP) {
+    for (int i = threadIdx.x; i < 64; i += OP_THREADS) hacc[i] = 0;
+    if (threadIdx.x < 2) hgrp[threadIdx.x] = -1;
+  }
+  LaneView<Real> L[2];
+  L[0] = lane_view<Real, IN, OUT>(a, T->l[0]);
+  L[1] = lane_view<Real, IN, OUT>(a, T->l[1]);
+  constexpr int U = 4;
+  for (int e0 = threadIdx.x; e0 < a.M; e0 += OP_THREADS * U) {
+    int nn[U];
+    Real v[2][U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) nn[u] = e0 + u * OP_THREADS < a.M ? e0 + u * OP_THREADS : -1;
+    gather_samples<Real, NS, IN, U>(a, L, nn, v);
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (nn[u] >= 0) buf[swz<SW>(nn[u])] = make_c<C, Real>(v[0][u], v[1][u]);
+  }
+  __syncthreads();
+  const Real* H = static_cast<const Real*>(a.H) + (long long)T->filter * a.M;
+  fft_rows_filter<C, SW>(buf, 1, rs, logM, tw, [H](int) { return H; });
+  for (int e0 = threadIdx.x; e0 < a.M; e0 += OP_THREADS * U) {   // M is a multiple of the threads
+    int nn[U];
+    Real val[2][U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      nn[u] = e0 + u * OP_THREADS < a.M ? e0 + u * OP_THREADS : -1;
+      C z = make_c<C, Real>(Real(0), Real(0));
+      if (nn[u] >= 0) z = buf[swz<SW>(nn[u])];
+      val[0][u] = c_re(z);
+      val[1][u] = c_im(z);
+    }
+    scatter_samples<Real, NS, OUT, U, (sizeof(Real) == 4 ? REG_RUN : 0)>(a, L, nn, val, hacc, hgrp);
+  }
+  if constexpr (HWP) {
+    if (a.hwp_base) {
+      __syncthreads();
+      for (int l = 0; l < 2; ++l)
+        hwp_flush(static_cast<Out*>(L[l].out), map_ns(NS) == 3 ? 4 : 1, hacc + 32 * l, hgrp + l, 1);
+    }
+  }
+}
+// Shared memory of k_one, and the most it may take (two CTAs per SM).
+template <typename Real>
+size_t smem_one(const Plan* p) {
+  const int logM = p->logN1 + p->logN2;
+  return (size_t)(lay_rs(sizeof(typename CxT<Real>::type), logM, false) + p->M) * sizeof(typename CxT<Real>::type);
+}
+constexpr size_t ONE_SMEM = (size_t)100 << 10;
+
 template <typename Real>
 inline int elems_per_cta() {
   return 1 << elog<Real>();
@@ -1593,6 +1677,8 @@ madmap_status launch_all(Plan* p, const void* in, void* out, long long in_stride
   a.tiles = ts ? ts->tiles : p->tiles;
   const int n_tiles = ts ? ts->n_tiles : p->n_tiles;
   const bool reg = p->reg.logN1 > 0;   // register transforms
+  const size_t sm1 = smem_one<Real>(p);
+  const bool one = !reg && sm1 <= ONE_SMEM;   // a tile per CTA
   const size_t sm13 = smem_f13<Real>(p), sm2 = smem_f2<Real>(p);
   const OpKernels K = pick_kernels<Real, NS, IN, OUT>(p);
   a.reg_logN1 = p->reg.logN1;
@@ -1602,7 +1688,9 @@ madmap_status launch_all(Plan* p, const void* in, void* out, long long in_stride
   a.reg_four0 = p->reg.four0;
   a.reg_wide = DF ? (const void*)p->wide_df : (const void*)p->wide64;
   // n_rhs == 0 only sets the kernels' attributes, so it can precede a capture
-  if (!reg) {
+  if (one) {
+    MM_CUDA(set_smem(k_one<Real, NS, IN, OUT>, sm1));
+  } else if (!reg) {
     MM_CUDA(set_smem(K.f1, sm13));
     MM_CUDA(set_smem(K.f3, sm13));
     MM_CUDA(set_smem(K.f2, sm2));
@@ -1693,6 +1781,13 @@ madmap_status launch_all(Plan* p, const void* in, void* out, long long in_stride
           if (st != MADMAP_OK) return st;
           continue;
         }
+        if (one) {
+          if (ev) cudaEventRecord(ev[ei++], cs);
+          k_one<Real, NS, IN, OUT><<<nt, OP_THREADS, sm1, cs>>>(a);
+          if (ev)
+            for (int k = 1; k < 4; ++k) cudaEventRecord(ev[ei++], cs);
+          continue;
+        }
         dim3 g13(p->N1 / a.B1, nt), g2(p->N2 / a.B2, nt);
         if (ev) cudaEventRecord(ev[ei++], s);
         K.f1<<<g13, OP_THREADS, sm13, cs>>>(a);
@@ -1720,7 +1815,7 @@ madmap_status launch_all(Plan* p, const void* in, void* out, long long in_stride
       MM_CUDA(cudaStreamWaitEvent(s, p->op_join[i], 0));
     }
   }
-  count_launches(3LL * n_chunks * n_rhs * reps);
+  count_launches((one ? 1LL : 3LL) * n_chunks * n_rhs * reps);
   MM_CUDA(cudaGetLastError());
   return MADMAP_OK;
 }

@@ -149,13 +149,6 @@ struct Powers {
   }
 };
 
-// Lanes of a run sum in k_c3 (run_sum): a run of samples in one pixel adds once
-// per aligned group of this many.  Four takes two shuffle steps of each of the
-// three sums where a warp row of 16 samples takes four, for one atomic in two
-// samples instead of one in three on the ring scan (0.65 repeats); the shuffles
-// were a third of the kernel's L1 wavefronts (16, 8, 4 lanes: 103.5, 97.9, 97.6
-// us per launch, 387, 377, 373 us per application).
-constexpr int REG_RUN = 4;
 // Columns per CTA of k_c1 and k_c3 (16 threads x 16 elements a column): 16 in
 // float32, at 64 registers and four CTAs per SM; 8 for the float64-size types,
 // at 128 registers and four CTAs of 128 threads.
