@@ -1146,8 +1146,11 @@ __global__ void __launch_bounds__(256, sizeof(Real) == 4 ? MM_MINB_F13 : MM_MINB
 // sums where a warp row of 16 samples takes four, for one atomic in two samples
 // instead of one in three on the ring scan (0.65 repeats); the shuffles were a
 // third of k_c3's L1 wavefronts (16, 8, 4 lanes: 103.5, 97.9, 97.6 us per launch,
-// 387, 377, 373 us per application).
-constexpr int REG_RUN = 4;
+// 387, 377, 373 us per application, the same error against 64 bits).
+#ifndef MM_RUN
+#define MM_RUN 4
+#endif
+constexpr int REG_RUN = MM_RUN;
 
 // ---------------------------------------------------------------- k_one
 // A whole tile in one CTA, for windows that fit its shared memory: gather, FFT,
@@ -1742,7 +1745,7 @@ madmap_status launch_all(Plan* p, const void* in, void* out, long long in_stride
   chunking(p, n_chunks, per_chunk, n_tiles, cap);
   // map replicas for small, heavily hit maps (single right-hand side per launch)
   typedef typename OutT<Real>::type Out;
-  const bool use_rep = !ts && OUT == OUT_MAP && p->n_rep > 1 && p->rep;
+  const bool use_rep = !ts && OUT == OUT_MAP && p->n_rep > 1 && p->rep && (sizeof(Real) == 4 || p->rep_wide);
   const long long n_map = (long long)std::max(1, p->n_obs) * p->ns_pad;
   // several chunks: alternate two streams (own scratch slot each) so chunks overlap
   // (with replicas only when one application is enqueued: the replicas are reused)

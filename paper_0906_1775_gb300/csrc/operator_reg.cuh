@@ -453,7 +453,7 @@ __global__ void __launch_bounds__(128, LA == 5 ? 2 : 4) k_xcorr(OpArgs a, double
 #pragma unroll
     for (int b = 0; b < RB; ++b) {
       const float2 u = za[q * RB + b], v = zr[q * RB + b];
-      atomicAdd(g + RB * q + RA * b, (double)u.x * (double)v.x + (double)u.y * (double)v.y);
+      atomicAdd(g + RB * q + RA * b, widen(u.x) * widen(v.x) + widen(u.y) * widen(v.y));
     }
 }
 

@@ -873,22 +873,36 @@ struct Seg {
   int out_lo, out_hi, filter;
 };
 
+// Windows of the register transforms (16 columns a CTA) over IQU pointing start
+// at multiples of 16 samples, so a warp's 16 samples of (pixel, angle) pairs are
+// one aligned 128-byte line instead of parts of two; up to 15 samples of a window
+// are spent on it (one application on the IQU raster, 97 tiles of 2^17: 201 -> 193
+// us, on the ring scan, 103 tiles of 2^18: 365 -> 361 us).  Temperature pointing is
+// half as wide and measured no different.
+constexpr int WINDOW_ALIGN = 16;
+static int window_align(int n_stokes, int n_lags, int M) {
+  return n_stokes == 3 && reg_log_n1(M) > 0 && M - 2LL * (n_lags - 1) >= 64 * WINDOW_ALIGN ? WINDOW_ALIGN : 1;
+}
+
+// align: windows start at multiples of this (window_align).
 static void make_segments(const std::vector<long long>& off, const std::vector<int>& filt, int n_lags, int M,
-                          std::vector<Seg>& segs) {
+                          int align, std::vector<Seg>& segs) {
   segs.clear();
-  const long long h = n_lags - 1;
-  const long long U = M - 2 * h;
+  const long long h = n_lags - 1, A = align;
+  const long long U = M - 2 * h - (A - 1);
+  auto down = [A](long long t) { return t >= 0 ? t / A * A : -((-t + A - 1) / A * A); };
   for (size_t i = 0; i + 1 < off.size(); ++i) {
     const long long t0 = off[i], t1 = off[i + 1], n = t1 - t0;
     if (n <= 0) continue;
-    if (n + h <= M) {
-      segs.push_back({t0, t0, t1, 0, (int)n, filt[i]});
+    if (n + h + (A - 1) <= M) {
+      const long long ws = down(t0), o = t0 - ws;
+      segs.push_back({ws, t0, t1, (int)o, (int)(o + n), filt[i]});
       continue;
     }
     for (long long u0 = t0; u0 < t1; u0 += U) {
       const long long u1 = std::min(t1, u0 + U);
-      const long long ws = u0 - h;
-      segs.push_back({ws, std::max(t0, ws), std::min(t1, ws + M), (int)h, (int)(h + u1 - u0), filt[i]});
+      const long long ws = down(u0 - h), o = u0 - ws;   // h <= o < h + A
+      segs.push_back({ws, std::max(t0, ws), std::min(t1, ws + M), (int)o, (int)(o + u1 - u0), filt[i]});
     }
   }
 }
@@ -931,7 +945,7 @@ static void pair_tiles(const std::vector<Seg>& segs, int n_filters, std::vector<
 void build_tiles(const std::vector<long long>& off, const std::vector<int>& filt, int n_filters, int n_lags, int M,
                  std::vector<Tile>& tiles) {
   std::vector<Seg> segs;
-  make_segments(off, filt, n_lags, M, segs);
+  make_segments(off, filt, n_lags, M, 1, segs);
   pair_tiles(segs, n_filters, tiles);
 }
 
@@ -991,7 +1005,7 @@ madmap_status get_tile_set(Plan* p, int n_rhs, TileSet** out) {
       return MADMAP_OK;
     }
   std::vector<Seg> segs;
-  make_segments(p->offsets, p->ivl_filter, p->n_lags, p->M, segs);
+  make_segments(p->offsets, p->ivl_filter, p->n_lags, p->M, window_align(p->n_stokes, p->n_lags, p->M), segs);
   std::vector<Tile> tiles;
   for (int f = 0; f < p->n_filters; ++f) {
     std::vector<std::pair<const Seg*, int>> lanes;
@@ -1057,7 +1071,7 @@ static int choose_fft_len(const std::vector<long long>& off, const std::vector<i
   for (int lg = 8; lg <= 20; ++lg) {
     const int M = 1 << lg;
     if (M - 2 * (n_lags - 1) < 1) continue;
-    make_segments(off, filt, n_lags, M, segs);
+    make_segments(off, filt, n_lags, M, 1, segs);
     pair_tiles(segs, n_filters, tiles);
     const double cost = (double)tiles.size() * (double)M * (lg + 8.0) + 1.0 * M;
     if (cost < best) {
@@ -1333,7 +1347,7 @@ static madmap_status setup_windows(Plan* p, int M, long long tpc_req, cudaStream
     p->N2 = 1 << p->logN2;
   }
   std::vector<Seg> segs;
-  make_segments(p->offsets, p->ivl_filter, p->n_lags, p->M, segs);
+  make_segments(p->offsets, p->ivl_filter, p->n_lags, p->M, window_align(p->n_stokes, p->n_lags, p->M), segs);
   p->host_tiles.clear();
   pair_tiles(segs, p->n_filters, p->host_tiles);
   p->n_segments = (int)segs.size();
@@ -1880,8 +1894,12 @@ extern "C" madmap_status madmap_plan_create(const madmap_plan_desc* d, void* str
     else
       MM_TRY(setup_windows(p, M0, d->tiles_per_chunk, s));
   }
-  if (!p->det && p->n_obs > 0 && p->n_t >= 1024LL * p->n_obs && (long long)p->n_obs * p->ns_pad <= (1LL << 17)) {
-    // a small map under more than 1024 samples per row: eight scatter replicas
+  if (!p->det && p->n_obs > 0 && p->n_t >= 200LL * p->n_obs && (long long)p->n_obs * p->ns_pad <= (1LL << 17)) {
+    // a small map under many samples: eight scatter replicas.  From 200 samples a
+    // row in float32 (64 x 64 map, 610 a row: application 58.8 -> 44.2 us; 64 a row:
+    // solve 1.02 -> 1.08 ms), from 1024 in float64 and double-float, whose
+    // transforms leave the atomics more time (610 a row: 351 -> 356 and 88 -> 92 us).
+    p->rep_wide = p->n_t >= 1024LL * p->n_obs;
     p->n_rep = 8;
     const size_t rb = sizeof(double) * (size_t)p->n_rep * p->n_obs * p->ns_pad;
     MM_TRY(dalloc(p, &p->rep, rb));

@@ -213,8 +213,8 @@ __device__ __forceinline__ void stv(Real* v, int p, const V3<Real, NS>& o) {
 }
 template <typename Real, int NS>
 __device__ __forceinline__ double dotv(const V3<Real, NS>& u, const V3<Real, NS>& v) {
-  double s = (double)u.a * (double)v.a;
-  if (NS == 3) s += (double)u.b * (double)v.b + (double)u.c * (double)v.c;
+  double s = widen(u.a) * widen(v.a);
+  if (NS == 3) s += widen(u.b) * widen(v.b) + widen(u.c) * widen(v.c);
   return s;
 }
 
