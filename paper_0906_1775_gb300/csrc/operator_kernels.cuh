@@ -1142,15 +1142,13 @@ __global__ void __launch_bounds__(256, sizeof(Real) == 4 ? MM_MINB_F13 : MM_MINB
 
 
 // Lanes of a run sum (run_sum): a run of samples in one pixel adds once per
-// aligned group of this many.  Four takes two shuffle steps of each of the three
-// sums where a warp row of 16 samples takes four, for one atomic in two samples
-// instead of one in three on the ring scan (0.65 repeats); the shuffles were a
-// third of k_c3's L1 wavefronts (16, 8, 4 lanes: 103.5, 97.9, 97.6 us per launch,
-// 387, 377, 373 us per application, the same error against 64 bits).
-#ifndef MM_RUN
-#define MM_RUN 4
-#endif
-constexpr int REG_RUN = MM_RUN;
+// aligned group of this many, here the 16 consecutive samples of a warp's row.
+// Shorter groups take fewer shuffles (a third of k_c3's L1 wavefronts on the ring
+// scan, 0.65 repeats: 16, 8 and 4 lanes take 103.5, 97.9 and 97.6 us per launch,
+// 387, 377 and 373 us per application) but more atomics, each a float32 rounding
+// in its pixel: the operator is 5.4e-7 to 6.3e-7 off 64 bits with 16 lanes and
+// 5.8e-7 to 7.6e-7 with 4.
+constexpr int REG_RUN = 16;
 
 // ---------------------------------------------------------------- k_one
 // A whole tile in one CTA, for windows that fit its shared memory: gather, FFT,

@@ -20,8 +20,7 @@
 // on half of 97 tiles of 2^17 (IQU, 512 x 512 raster): columns 67.7 -> 50.2 and
 // 61.5 -> 59.1 us, rows 30.9 -> 23.6 us, one application 262 -> 213 us; on 103
 // tiles of 2^18 (ring scan, N_side 512): 109 -> 77, 121 -> 112 and 65 -> 47 us,
-// 531 -> 412 us (and to 201 and 365 us with the packed sums and short run sums
-// below).  Sixteen columns a CTA because 256 threads x 16 elements leave
+// 531 -> 412 us (and to 201 and 387 us with the packed sums below).  Sixteen columns a CTA because 256 threads x 16 elements leave
 // four CTAs per SM at 64 registers; three CTAs with twice or four times the
 // loads in flight per thread measured slower (442 and 468 us on the ring scan),
 // and so did loading the pointing one to four batches ahead of the map (373 -> 387
