@@ -405,6 +405,17 @@ madmap_status madmap_plan_expand_pointing(madmap_plan_t plan, int32_t* pix, floa
  * recomputes spectra and preconditioner blocks.  Synchronises `stream`. */
 madmap_status madmap_plan_set_filters(madmap_plan_t plan, const double* filter_lags, void* stream);
 
+/* madmap_plan_set_filters with the lags that madmap_noise_filter gives for
+ * params (host [n_filters][3]: sigma, f_knee, alpha) at sample rate fs, formed on
+ * the device when n_lags is a power of two from 64 on. */
+madmap_status madmap_plan_set_noise(madmap_plan_t plan, double fs, const double* params, void* stream);
+
+/* The chain rule of madmap_noise_filter_vjp for all of a plan's filters:
+ * grad_lags (device [n_filters][n_lags]) -> grad_params (host [n_filters][3]).
+ * Synchronises `stream`. */
+madmap_status madmap_plan_noise_vjp(madmap_plan_t plan, double fs, const double* params, const double* grad_lags,
+                                    double* grad_params, void* stream);
+
 /* ------------------------------------------------------------------ operators */
 
 /* y = H x = A^T N^-1 A x (Eq. 10) for n_rhs maps.  x, y: device

@@ -536,6 +536,40 @@ class Plan:
     def set_filters(self, filter_lags, stream=None):
         madmap_plan_set_filters(self._h, np.atleast_2d(filter_lags), stream)
 
+    def _device_noise(self):
+        """Whether the library forms this lag count's noise filters on the device."""
+        n = self.stats["n_lags"]
+        return n >= 64 and n & (n - 1) == 0
+
+    def set_noise(self, fs, params, stream=None):
+        """Rebuild the filters from (sigma, f_knee, alpha) per filter (host [n_filters, 3])."""
+        prm = np.ascontiguousarray(params, dtype=np.float64)
+        if prm.shape != (self.stats["n_filters"], 3):
+            raise ValueError("params must be [n_filters, 3]")
+        if self._device_noise():
+            check(load().madmap_plan_set_noise(self._h, float(fs), prm.ctypes.data, C.c_void_p(_stream_ptr(stream))),
+                  "madmap_plan_set_noise")
+        else:   # other lag counts: one filter per host thread
+            self.set_filters(np.stack(_per_filter(
+                lambda k: madmap_noise_filter(self.stats["n_lags"], fs, *prm[k]), prm.shape[0])), stream)
+
+    def noise_vjp(self, fs, params, grad_lags, stream=None):
+        """Gradient of (sigma, f_knee, alpha) per filter (numpy [n_filters, 3]) from grad_lags, a float64 CUDA
+        tensor [n_filters, n_lags]."""
+        torch = _torch()
+        prm = np.ascontiguousarray(params, dtype=np.float64)
+        if prm.shape != (self.stats["n_filters"], 3):
+            raise ValueError("params must be [n_filters, 3]")
+        if not self._device_noise():
+            g = grad_lags.cpu().numpy()
+            return np.stack(_per_filter(
+                lambda k: madmap_noise_filter_vjp(self.stats["n_lags"], fs, *prm[k], g[k]), prm.shape[0]))
+        out = np.zeros_like(prm)
+        check(load().madmap_plan_noise_vjp(self._h, float(fs), prm.ctypes.data,
+                                           _dev_ptr(grad_lags, torch.float64, "grad_lags"), out.ctypes.data,
+                                           C.c_void_p(_stream_ptr(stream))), "madmap_plan_noise_vjp")
+        return out
+
     def _map_shape(self, n_rhs):
         return (n_rhs, self.n_obs, self.n_stokes)
 
@@ -715,9 +749,7 @@ def _autograd_function():
         @staticmethod
         def forward(ctx, d, params, plan, fs, solve_kwargs):
             prm = params.detach().cpu().numpy().astype(np.float64)
-            n_lags = plan.stats["n_lags"]
-            lags = np.stack(_per_filter(lambda k: madmap_noise_filter(n_lags, fs, *prm[k]), prm.shape[0]))
-            plan.set_filters(lags)
+            plan.set_noise(fs, prm)
             kw = dict(solve_kwargs or {})
             m, info = plan.solve(d.detach().contiguous(), **kw)
             ctx.save_for_backward(d, m, params)
@@ -738,10 +770,7 @@ def _autograd_function():
             gp = None
             if ctx.needs_input_grad[1]:
                 prm = params.detach().cpu().numpy().astype(np.float64)
-                glh = gl.cpu().numpy()
-                n_lags = plan.stats["n_lags"]
-                out = np.stack(_per_filter(lambda k: madmap_noise_filter_vjp(n_lags, ctx.fs, *prm[k], glh[k]),
-                                           prm.shape[0]))
+                out = plan.noise_vjp(ctx.fs, prm, gl)
                 gp = torch.from_numpy(out).to(dtype=params.dtype, device=params.device)
             return (gd.view_as(d) if gd is not None else None), gp, None, None, None
 

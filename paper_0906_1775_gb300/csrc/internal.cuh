@@ -356,6 +356,16 @@ struct CorrPlan {
   double* G = nullptr;           // [n_filters][256][M / 256]; NULL until set up
 };
 
+// Work buffers of the noise filters formed on the device (spectra.cu).
+struct NoiseBuffers {
+  const double2* tw = nullptr;   // [L], L = 4 n_lags
+  double2* scratch = nullptr;    // [batch][L]
+  double* x = nullptr;           // [n_filters][L / 2 + 1]
+  double* out = nullptr;         // [n_filters][n_lags]
+  double* prm = nullptr;         // [n_filters][3]; NULL until set up
+  int batch = 0;
+};
+
 // ---------------------------------------------------------------- plan
 struct SolveBuffers;  // solver.cu
 
@@ -465,6 +475,7 @@ struct Plan {
   // backward pass: timestreams A lambda and d - A m, lag-correlation work items
   float* bw_a = nullptr;           // [2 n_t]: a, then r
   CorrPlan corr;
+  NoiseBuffers noise;
   void* corr_items = nullptr;
   int n_corr_items = 0;
   // deterministic plans: the samples of every observed row in ascending order
@@ -596,6 +607,10 @@ bool corr_by_fft(const Plan* p);
 madmap_status corr_setup(Plan* p, cudaStream_t s);
 madmap_status corr_spectrum(Plan* p, cudaStream_t s);
 madmap_status corr_run(Plan* p, double* grad, cudaStream_t s);
+
+// Lags of noise parameters (host in and out) and their chain rule (spectra.cu).
+madmap_status noise_lags(Plan* p, double fs, const double* prm, double* lags, cudaStream_t s);
+madmap_status noise_vjp(Plan* p, double fs, const double* prm, const double* grad_lags, double* out, cudaStream_t s);
 
 // host FFT (radix 2, float64), for the noise filters and the allocation-free weighting
 void host_fft(std::vector<double>& re, std::vector<double>& im, bool inverse);

@@ -2025,3 +2025,11 @@ extern "C" madmap_status madmap_plan_set_filters(madmap_plan_t plan, const doubl
   // classify as excised again; every other pixel keeps its A^T A block.
   return build_preconditioner(p, s);
 }
+
+extern "C" madmap_status madmap_plan_set_noise(madmap_plan_t plan, double fs, const double* params, void* stream) {
+  MM_CHECK(plan && params, MADMAP_ERR_INVALID_ARG, "plan_set_noise: NULL argument");
+  Plan* p = reinterpret_cast<Plan*>(plan);
+  std::vector<double> lags((size_t)p->n_filters * p->n_lags);
+  const madmap_status st = noise_lags(p, fs, params, lags.data(), static_cast<cudaStream_t>(stream));
+  return st == MADMAP_OK ? madmap_plan_set_filters(plan, lags.data(), stream) : st;
+}

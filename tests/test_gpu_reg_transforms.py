@@ -82,3 +82,26 @@ def test_lag_gradient_matches_direct_correlation(lg):
     lam, _ = S.pcg(g, rel_tol=1e-13, max_iter=2000)
     scale = np.linalg.norm(S.unpoint(lam)) * np.linalg.norm(d64 - S.unpoint(host(m)))
     assert np.abs(host(gl) - ogl).max() < 4 * TOL * scale, np.abs(host(gl) - ogl).max() / scale
+
+
+@pytest.mark.parametrize("n_lags", [64, 100, 1024])
+def test_noise_filters_on_the_device_match_the_host(n_lags):
+    """set_noise and noise_vjp against madmap_noise_filter and its chain rule: the
+    same sums in float64 with another order, relative to the largest lag."""
+    import torch
+    import paper_0906_1775_gb300 as mm
+    prm = np.array([[1.0, 0.1, 2.0], [0.8, 5.0, 1.3], [1.2, 0.0, 1.0]])
+    p = tiny_T(seed=140, n=9000, width=8, n_lags=n_lags, ivls=(3000, 3000, 3000))
+    lags = np.stack([mm.noise_filter(n_lags, 100.0, *q) for q in prm])
+    args = (cuda(p.pix), None, p.n_pix, p.interval_offsets, [0, 1, 2])
+    plan, ref = mm.Plan(*args, np.ones((3, 1)) * (np.arange(n_lags) == 0)), mm.Plan(*args, lags)
+    plan.set_noise(100.0, prm)
+    y = cuda(np.random.default_rng(0).standard_normal(p.n_samples), torch.float64)
+    assert rel_rms(host(plan.apply_ninv(y)), host(ref.apply_ninv(y))) < 1e-13
+    g = np.random.default_rng(1).standard_normal((3, n_lags))
+    out = plan.noise_vjp(100.0, prm, cuda(g, torch.float64))
+    for k in range(3):
+        want = mm.madmap_noise_filter_vjp(n_lags, 100.0, *prm[k], g[k])
+        assert np.allclose(out[k], want, rtol=1e-11, atol=1e-11 * np.abs(want).max())
+    with pytest.raises(mm.MadmapError):
+        plan.set_noise(100.0, prm * np.array([-1.0, 1.0, 1.0]))
