@@ -1073,7 +1073,11 @@ static int choose_fft_len(const std::vector<long long>& off, const std::vector<i
     if (M - 2 * (n_lags - 1) < 1) continue;
     make_segments(off, filt, n_lags, M, 1, segs);
     pair_tiles(segs, n_filters, tiles);
-    const double cost = (double)tiles.size() * (double)M * (lg + 8.0) + 1.0 * M;
+    // lengths with neither register transforms nor one CTA per window (2^13, 2^19,
+    // 2^20) cost more per point: IQU operator of 4 x 2^20 samples and 300 lags at
+    // 2^13 71.8 us, at 2^14 61.4 us
+    const double path = reg_log_n1(M) > 0 || M <= 4096 ? 1.0 : 1.3;
+    const double cost = (double)tiles.size() * (double)M * (lg + 8.0) * path + 1.0 * M;
     if (cost < best) {
       best = cost;
       bestM = M;
