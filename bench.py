@@ -199,7 +199,7 @@ def operator_source_hash():
     import hashlib
     import re
     h = hashlib.sha256()
-    for f in ("operator_kernels.cuh", "internal.cuh"):
+    for f in ("operator_kernels.cuh", "operator_reg.cuh", "internal.cuh"):
         src = open(os.path.join(ROOT, "paper_0906_1775_gb300", "csrc", f)).read()
         src = re.sub(r"/\*.*?\*/", "", src, flags=re.S)
         src = re.sub(r"//[^\n]*", "", src)
@@ -870,7 +870,7 @@ def run_headline(args, world, rank, local):
                         "peak_source": f"{hbm_peak_src} hbm_gbs (MEASURED_PEAKS.json)"},
                 "t_roof_us": {"bytes": b_alg / (hbm_peak * 1e9) * 1e6, "flops": f_alg / (alu_peak * 1e12) * 1e6},
                 "per_kernel_ms": [float(x) for x in op_ms[:3]], "launches_per_application": [int(x) for x in op_launch],
-                "dominant_kernel": ["k_f1", "k_f2", "k_f3"][k_dom],
+                "dominant_kernel": ["k_c1", "k_c2", "k_c3"][k_dom],
                 "fp64_operator_ms": float(op64_ms[3]),
                 "df64_operator_ms": float(opdf_ms[3])}
     # DRAM traffic per application from the committed ncu summary, used only while

@@ -200,7 +200,7 @@ typedef struct {
    * to plan creation; ignored for white-noise plans. */
   int32_t autotune;
   /* Scatter of the float32 operator (stored T or IQU pointing, one
-   * pixelisation, atomic map sums, FFT lengths 2^13 .. 2^20): lanes holding
+   * pixelisation, atomic map sums): lanes holding
    * consecutive samples that hit one pixel add their sum with one atomic per
    * run instead of one per sample.  0 (default): on when at least a quarter
    * of the samples repeat their predecessor's pixel, or as the autotuner
@@ -210,7 +210,9 @@ typedef struct {
   /* Split of the FFT length into column and row transforms (the four-step
    * FFT, M = N1 N2): 0 (default) N2 = 2^ceil(log2(M) / 2), or as the
    * autotuner measures; 1: columns half as long, rows twice (N1 at most
-   * 1024).  Any split gives the same product up to rounding.  Must be 0 or 1. */
+   * 1024).  Any split gives the same product up to rounding.  Lengths 2^14 ..
+   * 2^18 run columns of 256 points, and windows small enough for one CTA no
+   * split, whatever the value.  Must be 0 or 1. */
   int32_t fft_split;
 } madmap_plan_desc;
 
@@ -221,7 +223,7 @@ typedef struct {
   int32_t n_fp64_pixels;   /* pixels keeping float64 preconditioner blocks */
   int32_t n_stokes;
   int32_t fft_len;         /* M */
-  int32_t n1, n2;          /* M = n1 * n2 (four-step factorisation) */
+  int32_t n1, n2;          /* M = n1 * n2 (nominal four-step factorisation; see fft_split) */
   int32_t n_segments;      /* overlap-save windows over all intervals */
   int32_t n_tiles;         /* window pairs (two real windows per complex FFT) */
   int32_t tiles_per_chunk;
@@ -237,7 +239,7 @@ typedef struct {
   int32_t n_hwp_params;    /* half-wave-plate parameters (32 per group; the last rows of the map) */
   int32_t n_excised_hwp;   /* half-wave-plate parameters without weight */
   int32_t n_map_replicas;  /* copies of the map the operator scatters into (8 for small maps under
-                              more than 1024 samples per row, else 1) */
+                              at least 200 samples per row, else 1) */
   int32_t deterministic;   /* 1 when map sums run in a fixed order (madmap_plan_desc.deterministic) */
   int32_t sharded;         /* 1 for a sharded plan (madmap_plan_desc.allreduce set) */
   int32_t n_tuned;         /* candidates the autotuner timed (0: not tuned), at most MADMAP_MAX_TUNED reported */

@@ -733,6 +733,14 @@ __host__ __device__ constexpr int lay_rs(int esz, int lg, bool cols) {
 // Threads per CTA of the operator kernels (every launch uses this many).
 constexpr int OP_THREADS = 256;
 
+// Shared memory of a whole window of M = 2^lg complex elements of esz bytes with
+// its twiddles, and the most that one CTA takes (k_one; two CTAs per SM).
+inline size_t one_smem(int esz, int lg) { return (size_t)(lay_rs(esz, lg, false) + (1 << lg)) * esz; }
+constexpr size_t ONE_SMEM = (size_t)100 << 10;
+inline bool one_cta(const Plan* p, int esz) {
+  return p->reg.logN1 == 0 && one_smem(esz, p->logN1 + p->logN2) <= ONE_SMEM;
+}
+
 // Multiplication by the constant w8^k = exp(-2 pi i k / 8), k = 0..3, or its
 // conjugate, written out so no general complex product is spent on it.
 template <int K, bool CONJ>

@@ -1227,14 +1227,6 @@ __global__ void __launch_bounds__(OP_THREADS, 2) k_one(OpArgs a) {
     }
   }
 }
-// Shared memory of k_one, and the most it may take (two CTAs per SM).
-template <typename Real>
-size_t smem_one(const Plan* p) {
-  const int logM = p->logN1 + p->logN2;
-  return (size_t)(lay_rs(sizeof(typename CxT<Real>::type), logM, false) + p->M) * sizeof(typename CxT<Real>::type);
-}
-constexpr size_t ONE_SMEM = (size_t)100 << 10;
-
 template <typename Real>
 inline int elems_per_cta() {
   return 1 << elog<Real>();
@@ -1687,8 +1679,8 @@ madmap_status launch_all(Plan* p, const void* in, void* out, long long in_stride
   a.tiles = ts ? ts->tiles : p->tiles;
   const int n_tiles = ts ? ts->n_tiles : p->n_tiles;
   const bool reg = p->reg.logN1 > 0;   // register transforms
-  const size_t sm1 = smem_one<Real>(p);
-  const bool one = !reg && sm1 <= ONE_SMEM;   // a tile per CTA
+  const size_t sm1 = one_smem(sizeof(typename CxT<Real>::type), p->logN1 + p->logN2);
+  const bool one = one_cta(p, sizeof(typename CxT<Real>::type));   // a tile per CTA
   const size_t sm13 = smem_f13<Real>(p), sm2 = smem_f2<Real>(p);
   const OpKernels K = pick_kernels<Real, NS, IN, OUT>(p);
   a.reg_logN1 = p->reg.logN1;

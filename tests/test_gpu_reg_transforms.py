@@ -1,7 +1,8 @@
-"""The float32 register transforms (window lengths 2^14 to 2^18).
+"""The operator by window length: one CTA per window (up to 2^12 points in
+float32, 2^11 in the wider types), the register transforms (2^14 to 2^18) and
+the three shared-memory kernels between and above.
 
-Every row length N1 = M / 256 of 64 to 1024 points runs its own kernel; the
-lengths just outside (2^13, 2^19) run the shared-memory ones.  Each length's
+Every row length N1 = M / 256 of 64 to 1024 points runs its own kernel.  Each length's
 N^-1 is checked against the Eq. 15 direct sum on intervals that end inside,
 at and past a window's exact part, and its operator (gather and scatter of both
 paired windows, an odd number of them, flagged samples) against the oracle.
@@ -22,13 +23,17 @@ from tests.helpers import lags_for, rel_rms, system_for, tiny_IQU, tiny_T
 pytestmark = pytest.mark.gpu
 
 TOL = 1e-6
+# the same count of roundings at 2^-53; double-float rounds at 2^-47 and passes
+# the two weights' products at that too
+TOLS = {"fp32": TOL, "fp64": TOL * 2.0 ** -29 * 4, "df64": TOL * 2.0 ** -23 * 4}
 
 
-@pytest.mark.parametrize("lg", range(13, 20))
+@pytest.mark.parametrize("lg", range(8, 20))
 def test_weighting_matches_direct_sum(lg):
     import torch
     from oracle.noise import apply_ninv_direct
-    M, n_lags = 1 << lg, 129
+    M = 1 << lg
+    n_lags = 129 if lg > 9 else 33
     exact = M - 2 * (n_lags - 1)     # samples one window weighs exactly
     p = tiny_T(seed=90 + lg, n=4 * exact + 777, width=24, n_lags=n_lags, ivls=(1, 775, exact, exact + 1, 2 * exact))
     plan = make_plan(p, fft_len=M)
@@ -42,19 +47,44 @@ def test_weighting_matches_direct_sum(lg):
         assert rel_rms(w[a:b], ref[a:b]) < 4 * TOL, i    # single samples carry no averaging
 
 
-@pytest.mark.parametrize("lg", range(14, 19))
-@pytest.mark.parametrize("runs", [-1, 1])
-def test_operator_matches_oracle(lg, runs):
-    import torch
+@pytest.fixture(scope="module")
+def flagged_iqu():
     p = tiny_IQU(seed=95, n_per_det=7001, n_lags=300, n_ivl_lo=200, n_ivl_hi=5000, flag_frac=0.02)
-    S = system_for(p)
+    return p, system_for(p)
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp64", "df64"])
+@pytest.mark.parametrize("lg", range(10, 19))
+@pytest.mark.parametrize("runs", [-1, 1])
+def test_operator_matches_oracle(flagged_iqu, lg, runs, prec):
+    import torch
+    p, S = flagged_iqu
+    if runs == 1 and prec != "fp32":
+        pytest.skip("run sums are float32")
     plan = make_plan(p, fft_len=1 << lg, scatter_runs=runs)
     x = np.random.default_rng(lg).standard_normal((S.n_obs, 3)).astype(np.float32)
     x[S.excised] = 0.0
-    y = host(plan.apply_ATNA(cuda(x, torch.float32), precision="fp32"))[0]
-    assert rel_rms(y, S.H(x.astype(np.float64))) < 2 * TOL   # two weights and a sum more per sample
-    b = host(plan.rhs(cuda(p.d), precision="fp32"))[0]
-    assert rel_rms(b, S.rhs(p.d[0])) < 2 * TOL
+    y = host(plan.apply_ATNA(cuda(x, torch.float32 if prec == "fp32" else torch.float64), precision=prec))[0]
+    assert rel_rms(y, S.H(x.astype(np.float64))) < 2 * TOLS[prec]   # two weights and a sum more per sample
+    b = host(plan.rhs(cuda(p.d), precision=prec))[0]
+    assert rel_rms(b, S.rhs(p.d[0])) < 2 * TOLS[prec]
+
+
+@pytest.mark.parametrize("width", [64, 65, 128, 129])
+@pytest.mark.parametrize("prec", ["fp64", "mixed"])
+def test_solve_around_the_cluster_kernel_s_map_sizes(width, prec):
+    """4096 rows fill its smaller form, 16384 its larger one; 129 x 129 rows run the
+    three vector kernels.  The same iterations give the oracle's map."""
+    p = tiny_T(seed=150 + width, n=6 * width * width, width=width, n_lags=8, ivls=(2 * width * width, 4 * width * width))
+    S = system_for(p)
+    plan = make_plan(p)
+    m, info = plan.solve(cuda(p.d[0]), precision=prec, rel_tol=1e-11, max_iter=200)
+    x, _ = S.solve(p.d[0], rel_tol=1e-13, max_iter=400)
+    assert info["status"] == 0 and rel_rms(host(m), x) < 1e-9
+    capped, i4 = plan.solve(cuda(p.d[0]), precision=prec, rel_tol=1e-30, max_iter=4)
+    assert i4["iters"] == 4 and i4["status"] == 1
+    two, infos = plan.solve_batched(cuda(np.concatenate([p.d, 2 * p.d])), precision=prec, rel_tol=1e-11, max_iter=200)
+    assert rel_rms(host(two[1]), 2 * x) < 1e-9 and infos[0]["status"] == 0
 
 
 @pytest.mark.parametrize("lg", [13, 14, 15, 16, 17, 18, 19])
