@@ -862,8 +862,8 @@ def run_headline(args, world, rank, local):
     k_dom = int(np.argmax(op_ms[:3] * op_launch))
     roofline = {"bound": "alu", "achieved": achieved_tf, "peak": alu_peak, "unit": "TFLOP/s",
                 "frac": achieved_tf / alu_peak, "traffic": None,
-                "kernel": "operator A^T N^-1 A, float32: one application = k_f1 (gather + column FFTs), "
-                          "k_f2 (row FFTs x filter), k_f3 (inverse column FFTs + scatter) over all tile chunks",
+                "kernel": "operator A^T N^-1 A, float32: one application = k_c1 (gather + column FFTs), "
+                          "k_c2 (row FFTs x filter), k_c3 (inverse column FFTs + scatter) over all tile chunks",
                 "alg_flops_per_launch": float(f_alg), "alg_bytes_per_launch": int(b_alg), "ms_per_launch": t_op,
                 "peak_source": f"{props.multi_processor_count} SMs x 128 FP32 lanes x 2 flops x {sm_mhz:.0f} MHz",
                 "hbm": {"achieved": achieved_gbs, "peak": hbm_peak, "unit": "GB/s", "frac": achieved_gbs / hbm_peak,

@@ -10,6 +10,7 @@
 //                   residual, best iterate, termination
 //   k_cg_direction  copy x to the best iterate if it improved, p = z + beta p,
 //                   q = 0
+// (maps of up to 16384 rows: k_cg_step does all three in one cluster).
 // Dot products are accumulated in float64 in every precision, per block, and
 // the last block to finish (atomic ticket, no waiting) reduces the partials in
 // a fixed order, so results are reproducible run to run.  All scalars live on
