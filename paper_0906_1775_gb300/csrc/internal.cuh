@@ -529,6 +529,11 @@ template <typename T>
 inline madmap_status dalloc_t(Plan* p, T** ptr, size_t count) {
   return dalloc(p, reinterpret_cast<void**>(ptr), count * sizeof(T));
 }
+// Copies a host array to the device on `s` and waits for it.  (A cudaMemcpy from
+// pageable memory may return before its last part is on the device, and only work
+// on the legacy stream and the streams that block with it would wait for that: not
+// the solves' stream, nor a caller's non-blocking one.)
+madmap_status upload(void* dst, const void* src, size_t bytes, cudaStream_t s);
 
 // ---------------------------------------------------------------- operator launch
 // Arithmetic of an operator application: float32, float64, or double-float
@@ -591,7 +596,7 @@ void build_tiles(const std::vector<long long>& off, const std::vector<int>& filt
                  std::vector<Tile>& tiles);
 
 // Tile set for n_rhs right-hand sides (cached in the plan).
-madmap_status get_tile_set(Plan* p, int n_rhs, TileSet** out);
+madmap_status get_tile_set(Plan* p, int n_rhs, TileSet** out, cudaStream_t s);
 
 // Deterministic plans: a timestream buffer for n_rhs right-hand sides.
 madmap_status ensure_wtod(Plan* p, int n_rhs);

@@ -52,6 +52,13 @@ madmap_status dalloc(Plan* p, void** ptr, size_t bytes) {
   return MADMAP_OK;
 }
 
+madmap_status upload(void* dst, const void* src, size_t bytes, cudaStream_t s) {
+  if (bytes == 0) return MADMAP_OK;
+  MM_CUDA(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, s));
+  MM_CUDA(cudaStreamSynchronize(s));
+  return MADMAP_OK;
+}
+
 // Device buffers that depend on the FFT length (windows, spectra, twiddles,
 // scratch): kept apart so the autotuner can rebuild them for another length.
 static madmap_status walloc(Plan* p, void** ptr, size_t bytes) {
@@ -994,7 +1001,7 @@ static madmap_status ensure_op_streams(Plan* p) {
   return MADMAP_OK;
 }
 
-madmap_status get_tile_set(Plan* p, int n_rhs, TileSet** out) {
+madmap_status get_tile_set(Plan* p, int n_rhs, TileSet** out, cudaStream_t s) {
   if (p->det) {
     madmap_status st = ensure_wtod(p, n_rhs);
     if (st != MADMAP_OK) return st;
@@ -1041,12 +1048,9 @@ madmap_status get_tile_set(Plan* p, int n_rhs, TileSet** out) {
     delete t;
     return st;
   }
-  if (!tiles.empty()) {
-    cudaError_t e = cudaMemcpy(t->tiles, tiles.data(), sizeof(Tile) * tiles.size(), cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) {
-      delete t;
-      return cuda_fail(e, "cudaMemcpy (tile set)");
-    }
+  if ((st = upload(t->tiles, tiles.data(), sizeof(Tile) * tiles.size(), s)) != MADMAP_OK) {
+    delete t;
+    return st;
   }
   if (!p->batch_tried && !p->tpc_fixed && t->n_tiles > p->tiles_per_chunk &&
       (size_t)p->tiles_per_chunk * p->M * sizeof(double2) < BATCH_SLOT_BYTES) {
@@ -1374,8 +1378,7 @@ static madmap_status setup_windows(Plan* p, int M, long long tpc_req, cudaStream
   }
   madmap_status st = walloc_t(p, &p->tiles, std::max(1, p->n_tiles));
   if (st != MADMAP_OK) return st;
-  if (p->n_tiles)
-    MM_CUDA(cudaMemcpy(p->tiles, p->host_tiles.data(), sizeof(Tile) * p->n_tiles, cudaMemcpyHostToDevice));
+  if ((st = upload(p->tiles, p->host_tiles.data(), sizeof(Tile) * p->n_tiles, s)) != MADMAP_OK) return st;
   if ((st = walloc_t(p, &p->H64, (size_t)p->n_filters * p->M)) != MADMAP_OK) return st;
   if ((st = walloc_t(p, &p->H32, (size_t)p->n_filters * p->M)) != MADMAP_OK) return st;
   if ((st = walloc_t(p, &p->Hdf, (size_t)p->n_filters * p->M)) != MADMAP_OK) return st;
@@ -1385,7 +1388,7 @@ static madmap_status setup_windows(Plan* p, int M, long long tpc_req, cudaStream
     std::vector<float> h(reg_table_floats(rl));
     reg_fill_tables(rl, h.data());
     if ((st = walloc_t(p, &tab, h.size())) != MADMAP_OK) return st;
-    MM_CUDA(cudaMemcpy(tab, h.data(), sizeof(float) * h.size(), cudaMemcpyHostToDevice));
+    if ((st = upload(tab, h.data(), sizeof(float) * h.size(), s)) != MADMAP_OK) return st;
     p->reg = reg_point_tables(rl, tab);
   }
   {
@@ -1403,9 +1406,9 @@ static madmap_status setup_windows(Plan* p, int M, long long tpc_req, cudaStream
     if ((st = walloc_t(p, &p->tw64, p->M)) != MADMAP_OK) return st;
     if (rl == 0 && (st = walloc_t(p, &p->tw32, p->M)) != MADMAP_OK) return st;
     if ((st = walloc_t(p, &p->twdf, p->M)) != MADMAP_OK) return st;
-    MM_CUDA(cudaMemcpy(p->tw64, t64.data(), sizeof(double2) * p->M, cudaMemcpyHostToDevice));
-    if (rl == 0) MM_CUDA(cudaMemcpy(p->tw32, t32.data(), sizeof(float2) * p->M, cudaMemcpyHostToDevice));
-    MM_CUDA(cudaMemcpy(p->twdf, tdf.data(), sizeof(cdf64) * p->M, cudaMemcpyHostToDevice));
+    if ((st = upload(p->tw64, t64.data(), sizeof(double2) * p->M, s)) != MADMAP_OK) return st;
+    if (rl == 0 && (st = upload(p->tw32, t32.data(), sizeof(float2) * p->M, s)) != MADMAP_OK) return st;
+    if ((st = upload(p->twdf, tdf.data(), sizeof(cdf64) * p->M, s)) != MADMAP_OK) return st;
     if (rl > 0) {
       const size_t n = (size_t)wide_four(rl) + p->M;
       if ((st = walloc_t(p, &p->wide64, n)) != MADMAP_OK) return st;
@@ -1858,12 +1861,11 @@ extern "C" madmap_status madmap_plan_create(const madmap_plan_desc* d, void* str
     p->n_diag_items = (int)items.size();
     MM_CHECK(items.size() < (1ULL << 31), MADMAP_ERR_INVALID_ARG, "too many samples for the white-noise pass");
     MM_TRY(dalloc_t(p, &p->diag_items, std::max<size_t>(1, items.size())));
-    if (!items.empty())
-      MM_TRYC(cudaMemcpy(p->diag_items, items.data(), sizeof(DiagItem) * items.size(), cudaMemcpyHostToDevice));
+    MM_TRY(upload(p->diag_items, items.data(), sizeof(DiagItem) * items.size(), s));
     std::vector<double> f0(p->n_filters);
     for (int f = 0; f < p->n_filters; ++f) f0[f] = p->lags[f];
     MM_TRY(dalloc_t(p, &p->f0_64, p->n_filters));
-    MM_TRYC(cudaMemcpy(p->f0_64, f0.data(), sizeof(double) * p->n_filters, cudaMemcpyHostToDevice));
+    MM_TRY(upload(p->f0_64, f0.data(), sizeof(double) * p->n_filters, s));
     p->diag = true;
   }
   // how often consecutive samples stay in one pixel: the scatter sums such
@@ -2022,7 +2024,7 @@ extern "C" madmap_status madmap_plan_set_filters(madmap_plan_t plan, const doubl
     return st;
   }
   if (p->diag) {  // the white-noise pass reads f(0) directly
-    MM_CUDA(cudaMemcpy(p->f0_64, p->lags.data(), sizeof(double) * p->n_filters, cudaMemcpyHostToDevice));
+    if ((st = upload(p->f0_64, p->lags.data(), sizeof(double) * p->n_filters, s)) != MADMAP_OK) return st;
   }
   // The block preconditioner weighs samples by f(0) of their filter: rebuild it.
   // Rows of excised pixels are already zero, so those pixels have no hits and

@@ -167,7 +167,9 @@ static madmap_status get_buffers(Plan* p, bool fp64, int n_rhs, SolveBuffers** o
     cudaError_t e = cudaMallocHost(&sb->host_st, 2 * sizeof(CgState) * n_rhs);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&sb->ev[0], cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&sb->ev[1], cudaEventDisableTiming);
+    // finished before any stream uses the buffers (the solves' stream does not wait for the legacy one)
     if (e == cudaSuccess) e = cudaMemset(sb->st, 0, sizeof(CgState) * n_rhs);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
     if (e != cudaSuccess) st = cuda_fail(e, "solve buffers");
   }
   slot = sb;  // freed with the plan, even when partially built
@@ -1384,7 +1386,7 @@ static madmap_status solve_impl(Plan* p, int n_rhs, const float* d, double* m, c
   B.n_rhs = n_rhs;
   if (n_rhs > 1) {
     TileSet* ts = nullptr;
-    madmap_status st = get_tile_set(p, n_rhs, &ts);
+    madmap_status st = get_tile_set(p, n_rhs, &ts, s);
     if (st != MADMAP_OK) return st;
     B.ts = ts;
   }
@@ -1703,8 +1705,7 @@ static madmap_status backward_impl(Plan* p, const float* d, const double* m, con
       CorrItem* dev = nullptr;
       st = dalloc(p, (void**)&dev, sizeof(CorrItem) * std::max<size_t>(1, items.size()));
       if (st != MADMAP_OK) return st;
-      if (!items.empty())
-        MM_CUDA(cudaMemcpy(dev, items.data(), sizeof(CorrItem) * items.size(), cudaMemcpyHostToDevice));
+      if ((st = upload(dev, items.data(), sizeof(CorrItem) * items.size(), s)) != MADMAP_OK) return st;
       p->corr_items = dev;
     }
     MM_CUDA(cudaMemsetAsync(grad_lags, 0, sizeof(double) * p->n_filters * p->n_lags, s));

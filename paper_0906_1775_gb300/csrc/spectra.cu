@@ -459,7 +459,7 @@ madmap_status corr_setup(Plan* p, cudaStream_t s) {
     reg_fill_tables(rl, h.data());
     float* tab = nullptr;
     if ((st = dalloc_t(p, &tab, h.size())) != MADMAP_OK) return st;
-    MM_CUDA(cudaMemcpy(tab, h.data(), sizeof(float) * h.size(), cudaMemcpyHostToDevice));
+    if ((st = upload(tab, h.data(), sizeof(float) * h.size(), s)) != MADMAP_OK) return st;
     c.reg = reg_point_tables(rl, tab);
     double2* tw = nullptr;
     if ((st = dalloc_t(p, &tw, M)) != MADMAP_OK) return st;
@@ -487,8 +487,7 @@ madmap_status corr_setup(Plan* p, cudaStream_t s) {
   c.per_chunk = (int)std::max<long long>(
       1, std::min<long long>(std::min<long long>(c.n_pairs, 32767), (long long)(CORR_SCRATCH / (2 * (size_t)M * sizeof(float2)))));
   if ((st = dalloc_t(p, &c.tiles, std::max<size_t>(1, both.size()))) != MADMAP_OK) return st;
-  if (!both.empty())
-    MM_CUDA(cudaMemcpy(c.tiles, both.data(), sizeof(Tile) * both.size(), cudaMemcpyHostToDevice));
+  if ((st = upload(c.tiles, both.data(), sizeof(Tile) * both.size(), s)) != MADMAP_OK) return st;
   // one buffer for the windows' transforms and then the float64 ones
   c.scratch_bytes = std::max((size_t)c.per_chunk * 2 * M * sizeof(float2), (size_t)M * sizeof(double2));
   if ((st = dalloc(p, &c.scratch, c.scratch_bytes)) != MADMAP_OK) return st;
