@@ -560,8 +560,10 @@ class Plan:
         prm = np.ascontiguousarray(params, dtype=np.float64)
         if prm.shape != (self.stats["n_filters"], 3):
             raise ValueError("params must be [n_filters, 3]")
+        if grad_lags.numel() != self.stats["n_filters"] * self.stats["n_lags"]:
+            raise ValueError("grad_lags must be [n_filters, n_lags]")
         if not self._device_noise():
-            g = grad_lags.cpu().numpy()
+            g = grad_lags.reshape(prm.shape[0], -1).cpu().numpy()
             return np.stack(_per_filter(
                 lambda k: madmap_noise_filter_vjp(self.stats["n_lags"], fs, *prm[k], g[k]), prm.shape[0]))
         out = np.zeros_like(prm)
