@@ -751,7 +751,7 @@ def _autograd_function():
         @staticmethod
         def forward(ctx, d, params, plan, fs, solve_kwargs):
             prm = params.detach().cpu().numpy().astype(np.float64)
-            plan.set_noise(fs, prm)
+            plan.set_noise(fs, prm[: plan.stats["n_filters"]])   # further rows have no filter
             kw = dict(solve_kwargs or {})
             m, info = plan.solve(d.detach().contiguous(), **kw)
             ctx.save_for_backward(d, m, params)
