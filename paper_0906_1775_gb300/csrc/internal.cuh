@@ -54,11 +54,11 @@ struct DiagItem {
   int filter, pad;
 };
 
-// Scratch of one launch of a tile set: four waves of the float32 column
+// The most scratch of one launch of a tile set: four waves of the float32 column
 // kernels' CTAs (152 SMs x 4 CTAs x 4096 elements) at 16 bytes an element.  A
-// set's own chunks instead of the plan's, which are sized for one right-hand
+// set has its own chunks instead of the plan's, which are sized for one right-hand
 // side (16 right-hand sides of 2.5e6 samples, M = 2^16: 31 launches of 208 CTAs
-// for 608 resident ones).
+// for 608 resident ones); smaller sets take what half of their tiles need.
 constexpr size_t BATCH_SLOT_BYTES = (size_t)4 * 152 * 4 * 4096 * 16;
 
 // A list of tiles whose lanes name their right-hand side (batched solves).
@@ -455,10 +455,10 @@ struct Plan {
   // each with its own scratch slot, so one chunk's kernels overlap the
   // previous chunk's tail and its scratch and pointing stay in L2.
   bool tpc_fixed = false;          // tiles_per_chunk set by the description
-  // Tile sets (batched solves) run in chunks of their own, two slots of
-  // BATCH_SLOT_BYTES allocated once by the first set larger than a plan chunk.
+  // Tile sets (batched solves) larger than a plan chunk run in chunks of their own,
+  // alternating two slots of batch_slot bytes that the largest set so far sized.
   void* batch_scratch = nullptr;
-  bool batch_tried = false;
+  size_t batch_slot = 0;
   cudaStream_t op_stream[2] = {nullptr, nullptr};
   cudaEvent_t op_fork = nullptr;
   cudaEvent_t op_join[2] = {nullptr, nullptr};
@@ -745,6 +745,9 @@ constexpr size_t ONE_SMEM = (size_t)100 << 10;
 inline bool one_cta(const Plan* p, int esz) {
   return p->reg.logN1 == 0 && one_smem(esz, p->logN1 + p->logN2) <= ONE_SMEM;
 }
+// Tiles of one launch of a tile set where scratch allows: at least two launches
+// from 16 tiles on, so that the two streams overlap.
+inline int set_chunk(int n_tiles) { return n_tiles >= 16 ? (n_tiles + 1) / 2 : n_tiles; }
 
 // Multiplication by the constant w8^k = exp(-2 pi i k / 8), k = 0..3, or its
 // conjugate, written out so no general complex product is spent on it.

@@ -1728,17 +1728,22 @@ madmap_status launch_all(Plan* p, const void* in, void* out, long long in_stride
     MM_CUDA(cudaGetLastError());
     return MADMAP_OK;
   }
-  // scratch slots of this launch: the plan's, or a tile set's own (at least
-  // two chunks from 16 tiles on, so that the two streams overlap)
+  // scratch slots of this launch: the plan's, or those of the tile sets larger than
+  // a plan chunk (k_one needs none)
   char* scratch = static_cast<char*>(p->scratch);
   size_t slot_bytes = (size_t)p->tiles_per_chunk * p->M * sizeof(double2);
   int slots = p->scratch_slots, cap = 0;
-  if (ts && p->batch_scratch) {
-    scratch = static_cast<char*>(p->batch_scratch);
-    slot_bytes = BATCH_SLOT_BYTES;
-    slots = 2;
-    cap = (int)std::min<size_t>(slot_bytes / ((size_t)p->M * sizeof(typename CxT<Real>::type)), 65535);
-    if (n_tiles >= 16) cap = std::min(cap, (n_tiles + 1) / 2);
+  if (ts && !p->tpc_fixed && n_tiles > p->tiles_per_chunk && p->op_fork) {
+    if (one) {
+      slots = 2;
+      cap = set_chunk(n_tiles);
+    } else if (p->batch_scratch && (slots < 2 || p->batch_slot > slot_bytes)) {
+      scratch = static_cast<char*>(p->batch_scratch);
+      slot_bytes = p->batch_slot;
+      slots = 2;
+      cap = (int)std::min<size_t>(slot_bytes / ((size_t)p->M * sizeof(typename CxT<Real>::type)), 65535);
+      cap = std::min(cap, set_chunk(n_tiles));
+    }
   }
   int n_chunks, per_chunk;
   chunking(p, n_chunks, per_chunk, n_tiles, cap);
@@ -1748,7 +1753,7 @@ madmap_status launch_all(Plan* p, const void* in, void* out, long long in_stride
   const long long n_map = (long long)std::max(1, p->n_obs) * p->ns_pad;
   // several chunks: alternate two streams (own scratch slot each) so chunks overlap
   // (with replicas only when one application is enqueued: the replicas are reused)
-  const bool pipe = !ev && n_rhs > 0 && n_chunks > 1 && p->op_stream[0] && slots > 1 &&
+  const bool pipe = !ev && n_rhs > 0 && n_chunks > 1 && p->op_fork && slots > 1 &&
                     (!use_rep || n_rhs * reps == 1);
   const int rgrid = (int)std::min<long long>((n_map + 255) / 256, 152LL * 8);
   if (pipe) {

@@ -95,6 +95,7 @@ static void free_windows(Plan* p) {
 }
 
 void free_solve_buffers(Plan* p);          // solver.cu
+void drop_solve_graphs(Plan* p);           // solver.cu
 size_t solve_buffer_bytes(const Plan* p);  // solver.cu
 
 Plan::~Plan() {
@@ -992,13 +993,39 @@ static madmap_status build_det_rows(Plan* p, cudaStream_t s) {
 
 // The two streams (and their events) that chunks alternate between.
 static madmap_status ensure_op_streams(Plan* p) {
-  if (p->op_stream[0]) return MADMAP_OK;
+  if (p->op_fork) return MADMAP_OK;   // created last
   for (int i = 0; i < 2; ++i) {
-    MM_CUDA(cudaStreamCreateWithFlags(&p->op_stream[i], cudaStreamNonBlocking));
-    MM_CUDA(cudaEventCreateWithFlags(&p->op_join[i], cudaEventDisableTiming));
+    if (!p->op_stream[i]) MM_CUDA(cudaStreamCreateWithFlags(&p->op_stream[i], cudaStreamNonBlocking));
+    if (!p->op_join[i]) MM_CUDA(cudaEventCreateWithFlags(&p->op_join[i], cudaEventDisableTiming));
   }
   MM_CUDA(cudaEventCreateWithFlags(&p->op_fork, cudaEventDisableTiming));
   return MADMAP_OK;
+}
+
+// Scratch of a set of n_tiles tiles larger than a plan chunk: as much as its
+// launches take, at most BATCH_SLOT_BYTES each.  Without the memory the set runs in
+// what is there: an earlier set's slots, or the plan's chunks.
+static void ensure_batch_scratch(Plan* p, int n_tiles) {
+  if (p->tpc_fixed || n_tiles <= p->tiles_per_chunk) return;
+  if (ensure_op_streams(p) != MADMAP_OK) {
+    cudaGetLastError();
+    return;
+  }
+  if (one_cta(p, sizeof(float2)) && one_cta(p, sizeof(double2))) return;   // no scratch
+  const size_t tile = (size_t)p->M * sizeof(double2);
+  const size_t want = std::min((size_t)set_chunk(n_tiles) * tile, std::max(tile, BATCH_SLOT_BYTES / tile * tile));
+  if (want <= p->batch_slot || (p->scratch_slots > 1 && want <= (size_t)p->tiles_per_chunk * tile)) return;
+  void* buf = nullptr;
+  if (dalloc(p, &buf, 2 * want) != MADMAP_OK) return;
+  if (p->batch_scratch) {   // the captured loops of earlier sets point into it
+    cudaDeviceSynchronize();
+    drop_solve_graphs(p);
+    cudaFree(p->batch_scratch);
+    p->allocs.erase(std::find(p->allocs.begin(), p->allocs.end(), p->batch_scratch));
+    p->device_bytes -= 2 * p->batch_slot;
+  }
+  p->batch_scratch = buf;
+  p->batch_slot = want;
 }
 
 madmap_status get_tile_set(Plan* p, int n_rhs, TileSet** out, cudaStream_t s) {
@@ -1052,13 +1079,7 @@ madmap_status get_tile_set(Plan* p, int n_rhs, TileSet** out, cudaStream_t s) {
     delete t;
     return st;
   }
-  if (!p->batch_tried && !p->tpc_fixed && t->n_tiles > p->tiles_per_chunk &&
-      (size_t)p->tiles_per_chunk * p->M * sizeof(double2) < BATCH_SLOT_BYTES) {
-    // larger chunks for tile sets; without the memory they run in the plan's
-    p->batch_tried = true;
-    if (ensure_op_streams(p) == MADMAP_OK && dalloc(p, &p->batch_scratch, 2 * BATCH_SLOT_BYTES) != MADMAP_OK)
-      p->batch_scratch = nullptr;
-  }
+  ensure_batch_scratch(p, t->n_tiles);
   p->tile_sets.push_back(t);
   *out = t;
   return MADMAP_OK;

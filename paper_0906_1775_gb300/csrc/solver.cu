@@ -97,11 +97,17 @@ static int grid_vec(long long n) {
   return (int)std::max(1LL, std::min<long long>(g, NB));
 }
 
-static void free_one(SolveBuffers* sb) {
-  if (!sb) return;
+static void drop_graphs(SolveBuffers* sb) {
   if (sb->exec) cudaGraphExecDestroy(sb->exec);
   if (sb->wexec) cudaGraphExecDestroy(sb->wexec);
   if (sb->wgraph) cudaGraphDestroy(sb->wgraph);
+  sb->exec = sb->wexec = nullptr;
+  sb->wgraph = nullptr;
+}
+
+static void free_one(SolveBuffers* sb) {
+  if (!sb) return;
+  drop_graphs(sb);
   for (int i = 0; i < 2; ++i)
     if (sb->ev[i]) cudaEventDestroy(sb->ev[i]);
   if (sb->host_st) cudaFreeHost(sb->host_st);
@@ -111,6 +117,12 @@ static void free_one(SolveBuffers* sb) {
 
 size_t solve_buffer_bytes(const Plan* p) {
   return (p->sb64 ? p->sb64->bytes : 0) + (p->sb32 ? p->sb32->bytes : 0);
+}
+
+// The captured loops, which are captured again when next needed.
+void drop_solve_graphs(Plan* p) {
+  if (p->sb32) drop_graphs(p->sb32);
+  if (p->sb64) drop_graphs(p->sb64);
 }
 
 void free_solve_buffers(Plan* p) {
