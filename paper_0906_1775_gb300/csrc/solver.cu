@@ -184,8 +184,11 @@ static madmap_status get_buffers(Plan* p, bool fp64, int n_rhs, SolveBuffers** o
     if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
     if (e != cudaSuccess) st = cuda_fail(e, "solve buffers");
   }
-  slot = sb;  // freed with the plan, even when partially built
-  if (st != MADMAP_OK) return st;
+  if (st != MADMAP_OK) {   // nothing half built is left for the next call
+    free_one(sb);
+    return st;
+  }
+  slot = sb;
   *out = sb;
   return MADMAP_OK;
 }
