@@ -1706,9 +1706,13 @@ static madmap_status backward_impl(Plan* p, const float* d, const double* m, con
     st = op_launch(p, false, IN_TOD_REAL, OUT_TOD, p->bw_a, grad_d, 0, 0, 1, nullptr, s);
     if (st != MADMAP_OK) return st;
   }
-  if (grad_lags && corr_by_fft(p)) {
-    if ((st = corr_setup(p, s)) != MADMAP_OK || (st = corr_run(p, grad_lags, s)) != MADMAP_OK) return st;
-  } else if (grad_lags) {
+  bool by_fft = grad_lags && corr_by_fft(p);
+  if (by_fft) {
+    st = corr_setup(p, s);
+    by_fft = st != MADMAP_ERR_OOM;   // the direct sums need only their item list
+    if (by_fft && (st != MADMAP_OK || (st = corr_run(p, grad_lags, s)) != MADMAP_OK)) return st;
+  }
+  if (grad_lags && !by_fft) {
     if (!p->corr_items) {
       std::vector<CorrItem> items;
       const long long chunk = 65536;

@@ -316,7 +316,8 @@ madmap_status build_spectra(Plan* p, cudaStream_t s) {
 
 // ---------------------------------------------------------------- noise filters from their parameters
 // madmap_noise_filter and its chain rule for all of a plan's filters at once, for
-// lag counts whose grid of L = 4 n_lags frequencies the transforms take.  8 filters
+// lag counts whose grid of L = 4 n_lags frequencies the transforms take (on the host,
+// filter by filter, where the device has no memory left for it).  8 filters
 // of 4096 lags on host threads: 2.2 ms and 2.3 ms a training step.
 namespace {
 
@@ -327,19 +328,19 @@ bool noise_on_device(const Plan* p) {
 madmap_status noise_setup(Plan* p, cudaStream_t s) {
   NoiseBuffers& b = p->noise;
   if (b.prm) return MADMAP_OK;
-  const int L = 4 * p->n_lags, F = p->n_filters;
-  madmap_status st = MADMAP_OK;
-  double2* tw = nullptr;
-  b.batch = (int)std::max<long long>(1, std::min<long long>(F, ((long long)64 << 20) / (16LL * L)));
-  if ((st = dalloc_t(p, &tw, L)) != MADMAP_OK || (st = dalloc_t(p, &b.scratch, (size_t)b.batch * L)) != MADMAP_OK ||
-      (st = dalloc_t(p, &b.x, (size_t)F * (L / 2 + 1))) != MADMAP_OK ||
-      (st = dalloc_t(p, &b.out, (size_t)F * p->n_lags)) != MADMAP_OK)
-    return st;
-  k_fill_twiddles<<<(L + 255) / 256, 256, 0, s>>>(tw, L);
-  b.tw = tw;
-  double* prm = nullptr;
-  if ((st = dalloc_t(p, &prm, (size_t)3 * F)) != MADMAP_OK) return st;
-  b.prm = prm;   // set last: the setup is complete
+  const size_t L = 4 * (size_t)p->n_lags, F = (size_t)p->n_filters;
+  b.batch = (int)std::max<size_t>(1, std::min<size_t>(F, ((size_t)64 << 20) / (16 * L)));
+  // one allocation: all of it or, for the host's sums, none
+  const size_t n_x = F * (L / 2 + 1), n_out = F * p->n_lags;
+  double2* base = nullptr;
+  const madmap_status st = dalloc_t(p, &base, (b.batch + 1) * L + (n_x + n_out + 3 * F + 1) / 2);
+  if (st != MADMAP_OK) return st;
+  b.scratch = base + L;
+  b.x = reinterpret_cast<double*>(b.scratch + b.batch * L);
+  b.out = b.x + n_x;
+  k_fill_twiddles<<<(int)((L + 255) / 256), 256, 0, s>>>(base, (int)L);
+  b.tw = base;
+  b.prm = b.out + n_out;   // set last: the setup is complete
   return MADMAP_OK;
 }
 
@@ -371,12 +372,13 @@ madmap_status noise_lags(Plan* p, double fs, const double* prm, double* lags, cu
   madmap_status st = check_noise(p, fs, prm);
   if (st != MADMAP_OK) return st;
   const size_t F = (size_t)p->n_filters;
-  if (!noise_on_device(p)) {
+  if (!noise_on_device(p) || (st = noise_setup(p, s)) == MADMAP_ERR_OOM) {
+    st = MADMAP_OK;
     for (size_t f = 0; f < F && st == MADMAP_OK; ++f)
       st = madmap_noise_filter(p->n_lags, fs, prm[3 * f], prm[3 * f + 1], prm[3 * f + 2], lags + f * p->n_lags, nullptr);
     return st;
   }
-  if ((st = noise_setup(p, s)) != MADMAP_OK) return st;
+  if (st != MADMAP_OK) return st;
   MM_CUDA(cudaMemcpyAsync(p->noise.prm, prm, sizeof(double) * 3 * F, cudaMemcpyHostToDevice, s));
   SpecArgs a = noise_args(p, fs);
   const long long n = (long long)F * (a.M / 2 + 1);
@@ -396,7 +398,8 @@ madmap_status noise_vjp(Plan* p, double fs, const double* prm, const double* gra
   madmap_status st = check_noise(p, fs, prm);
   if (st != MADMAP_OK) return st;
   const size_t F = (size_t)p->n_filters;
-  if (!noise_on_device(p)) {
+  if (!noise_on_device(p) || (st = noise_setup(p, s)) == MADMAP_ERR_OOM) {
+    st = MADMAP_OK;
     std::vector<double> g(F * p->n_lags);
     MM_CUDA(cudaMemcpyAsync(g.data(), grad_lags, sizeof(double) * g.size(), cudaMemcpyDeviceToHost, s));
     MM_CUDA(cudaStreamSynchronize(s));
@@ -405,7 +408,7 @@ madmap_status noise_vjp(Plan* p, double fs, const double* prm, const double* gra
                                    out + 3 * f);
     return st;
   }
-  if ((st = noise_setup(p, s)) != MADMAP_OK) return st;
+  if (st != MADMAP_OK) return st;
   MM_CUDA(cudaMemcpyAsync(p->noise.prm, prm, sizeof(double) * 3 * F, cudaMemcpyHostToDevice, s));
   SpecArgs a = noise_args(p, fs);
   a.x = grad_lags;
@@ -454,21 +457,6 @@ madmap_status corr_setup(Plan* p, cudaStream_t s) {
   const int rl = reg_log_n1(M), lg = rl + 8;
   c.logN2 = (lg + 1) / 2;
   c.logN1 = lg - c.logN2;
-  if (own) {
-    std::vector<float> h(reg_table_floats(rl));
-    reg_fill_tables(rl, h.data());
-    float* tab = nullptr;
-    if ((st = dalloc_t(p, &tab, h.size())) != MADMAP_OK) return st;
-    if ((st = upload(tab, h.data(), sizeof(float) * h.size(), s)) != MADMAP_OK) return st;
-    c.reg = reg_point_tables(rl, tab);
-    double2* tw = nullptr;
-    if ((st = dalloc_t(p, &tw, M)) != MADMAP_OK) return st;
-    k_fill_twiddles<<<(M + 255) / 256, 256, 0, s>>>(tw, M);
-    c.tw = tw;
-  } else {
-    c.reg = p->reg;
-    c.tw = p->tw64;
-  }
   // window pairs, each twice: a at the exact outputs (rhs 0), r over the input (rhs 1)
   std::vector<Tile> tiles, both;
   build_tiles(p->offsets, p->ivl_filter, p->n_filters, p->n_lags, M, tiles);
@@ -486,18 +474,40 @@ madmap_status corr_setup(Plan* p, cudaStream_t s) {
   c.n_pairs = (int)tiles.size();
   c.per_chunk = (int)std::max<long long>(
       1, std::min<long long>(std::min<long long>(c.n_pairs, 32767), (long long)(CORR_SCRATCH / (2 * (size_t)M * sizeof(float2)))));
-  if ((st = dalloc_t(p, &c.tiles, std::max<size_t>(1, both.size()))) != MADMAP_OK) return st;
-  if ((st = upload(c.tiles, both.data(), sizeof(Tile) * both.size(), s)) != MADMAP_OK) return st;
   // one buffer for the windows' transforms and then the float64 ones
   c.scratch_bytes = std::max((size_t)c.per_chunk * 2 * M * sizeof(float2), (size_t)M * sizeof(double2));
-  if ((st = dalloc(p, &c.scratch, c.scratch_bytes)) != MADMAP_OK) return st;
-  double* G = nullptr;
-  if ((st = dalloc_t(p, &G, (size_t)p->n_filters * M)) != MADMAP_OK) return st;
-  c.G = G;   // set last: the setup is complete
+  // one allocation: all of it or, for the direct sums, none
+  std::vector<float> h(own ? reg_table_floats(rl) : 0);
+  size_t bytes = 0;
+  auto part = [&bytes](size_t n) {
+    const size_t o = bytes;
+    bytes = (o + n + 255) & ~(size_t)255;
+    return o;
+  };
+  const size_t o_scratch = part(c.scratch_bytes), o_G = part((size_t)p->n_filters * M * sizeof(double)),
+               o_tiles = part(both.size() * sizeof(Tile)), o_tw = part(own ? (size_t)M * sizeof(double2) : 0),
+               o_tab = part(h.size() * sizeof(float));
+  char* base = nullptr;
+  if ((st = dalloc_t(p, &base, bytes)) != MADMAP_OK) return st;
+  c.scratch = base + o_scratch;
+  c.tiles = reinterpret_cast<Tile*>(base + o_tiles);
+  if ((st = upload(c.tiles, both.data(), sizeof(Tile) * both.size(), s)) != MADMAP_OK) return st;
+  if (own) {
+    reg_fill_tables(rl, h.data());
+    if ((st = upload(base + o_tab, h.data(), sizeof(float) * h.size(), s)) != MADMAP_OK) return st;
+    c.reg = reg_point_tables(rl, reinterpret_cast<const float*>(base + o_tab));
+    double2* tw = reinterpret_cast<double2*>(base + o_tw);
+    k_fill_twiddles<<<(M + 255) / 256, 256, 0, s>>>(tw, M);
+    c.tw = tw;
+  } else {
+    c.reg = p->reg;
+    c.tw = p->tw64;
+  }
+  c.G = reinterpret_cast<double*>(base + o_G);   // set last: the setup is complete
   return MADMAP_OK;
 }
 
-// grad[filter][tau] from p->bw_a and p->bw_r (corr_setup done).
+// grad[filter][tau] from p->bw_a, a and then r (corr_setup done).
 madmap_status corr_run(Plan* p, double* grad, cudaStream_t s) {
   CorrPlan& c = p->corr;
   MM_CUDA(cudaMemsetAsync(c.G, 0, sizeof(double) * (size_t)p->n_filters * c.M, s));

@@ -73,3 +73,36 @@ m2, _ = make_plan(p).solve(d, **kw)
 assert info["status"] == 0 and rel_rms(host(m), host(m2)) < 1e-8
 print("DONE")
 ''' % nth)
+
+
+def test_lag_gradient_and_noise_filters_do_without_their_buffers():
+    """The transforms' buffers refused: direct sums; the noise filters' refused: the host's sums."""
+    _run(r'''
+def set_up():
+    plan = make_plan(p)
+    m, _ = plan.solve(d, **kw)
+    g = torch.ones_like(m)
+    plan.solve_backward(d, m, g, want_lags=False, **kw)
+    return plan, m, g
+(plan, m, g), n = refuse_each(set_up)
+assert n > 30
+os.environ[VAR] = str(count + 1)
+_, gl, _ = plan.solve_backward(d, m, g, want_d=False, **kw)
+count += 2                                     # the refused buffers, and the direct sums' item list
+prm = np.array([[1.1, 3.0, 1.2]])
+os.environ[VAR] = str(count + 1)
+plan.set_noise(p.fs, prm)
+del os.environ[VAR]
+fresh = make_plan(p)
+_, gl2, _ = fresh.solve_backward(d, m, g, want_d=False, **kw)
+# a lag is an inner product of a = A lambda and a shifted r = d - A m, and each way of
+# summing it in float32 is within 4e-6 |a| |r| of it (test_gpu_reg_transforms)
+S = system_for(p)
+lam, _ = S.pcg(host(g), rel_tol=1e-13, max_iter=1000)
+scale = np.linalg.norm(S.unpoint(lam)) * np.linalg.norm(p.d[0] - S.unpoint(host(m)))
+assert np.abs(host(gl) - host(gl2)).max() < 8e-6 * scale, np.abs(host(gl) - host(gl2)).max() / scale
+other = make_plan(p, lags=mm.noise_filter(p.n_lags, p.fs, *prm[0])[None])
+y = cuda(np.random.default_rng(0).standard_normal(p.n_samples), torch.float64)
+assert rel_rms(host(plan.apply_ninv(y)), host(other.apply_ninv(y))) < 1e-12
+print("DONE")
+''')
