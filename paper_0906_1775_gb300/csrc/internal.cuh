@@ -346,6 +346,7 @@ RegTables reg_point_tables(int logN1, const float* base);
 // Lag correlation of the backward pass by transforms (spectra.cu): windows of
 // length M in pairs, each pair twice (a, then r), and the cross spectra.
 struct CorrPlan {
+  int route = 0;                 // 1: transforms, 2: direct sums (corr_by_fft; 0: not chosen yet)
   int M = 0, logN1 = 0, logN2 = 0;
   RegTables reg;
   const double2* tw = nullptr;   // [M]
@@ -606,9 +607,11 @@ madmap_status build_spectra(Plan* p, cudaStream_t s);
 // The wide register tables of p->M from tw64 and twdf (spectra.cu).
 madmap_status fill_wide_tables(Plan* p, cudaStream_t s);
 
-// Backward pass: lag correlation of p->bw_a by transforms where corr_by_fft;
+// Backward pass: lag correlation of p->bw_a by transforms where corr_by_fft, else by
+// direct sums (k_lag_corr: blocks of CORR_LB lags, items of CORR_CHUNK samples);
 // corr_spectrum (operator_f32.cu) sums the windows' cross spectra into corr.G.
-bool corr_by_fft(const Plan* p);
+constexpr int CORR_LB = 2048, CORR_CHUNK = 65536;
+bool corr_by_fft(Plan* p);
 madmap_status corr_setup(Plan* p, cudaStream_t s);
 madmap_status corr_spectrum(Plan* p, cudaStream_t s);
 madmap_status corr_run(Plan* p, double* grad, cudaStream_t s);

@@ -1586,8 +1586,8 @@ __global__ void k_mask_excised(double* b, long long nvec_pixels, int ns_pad, con
   }
 }
 
-// Lag correlation sum_{|t-t'|=tau} a_t r_t' by direct sums, for more lags than
-// the transforms of spectra.cu take windows for (corr_by_fft): CTA (lag block,
+// Lag correlation sum_{|t-t'|=tau} a_t r_t' by direct sums, for short intervals and
+// for more lags than the transforms of spectra.cu take (corr_by_fft): CTA (lag block,
 // work item) covers CORR_LB lags over the samples [t_lo, t_hi) of one
 // interval, in tiles of CORR_TT samples staged in shared memory, and adds
 // its totals to grad[filter][tau] (float64 atomics, one per lag and item).
@@ -1606,7 +1606,7 @@ struct CorrItem {
 // float64 across tiles and items.
 constexpr int CORR_R = 8;
 constexpr int CORR_T = 256;
-constexpr int CORR_LB = CORR_R * CORR_T;  // lags per block
+static_assert(CORR_LB == CORR_R * CORR_T, "lags per block");
 constexpr int CORR_TT = 1024;             // samples per tile
 constexpr int CORR_W = CORR_TT + CORR_LB;
 __device__ __forceinline__ int cpad(int i) { return i + (i >> 3); }
@@ -1715,7 +1715,7 @@ static madmap_status backward_impl(Plan* p, const float* d, const double* m, con
   if (grad_lags && !by_fft) {
     if (!p->corr_items) {
       std::vector<CorrItem> items;
-      const long long chunk = 65536;
+      const long long chunk = CORR_CHUNK;
       for (int i = 0; i < p->n_ivl; ++i)
         for (long long t = p->offsets[i]; t < p->offsets[i + 1]; t += chunk)
           items.push_back({p->offsets[i], p->offsets[i + 1], t, std::min(p->offsets[i + 1], t + chunk),

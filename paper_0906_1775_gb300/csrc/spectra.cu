@@ -439,20 +439,57 @@ madmap_status noise_vjp(Plan* p, double fs, const double* prm, const double* gra
 static constexpr int CORR_MAX_LAGS = 3 << 15;
 static constexpr size_t CORR_SCRATCH = (size_t)128 << 20;
 
-bool corr_by_fft(const Plan* p) { return p->n_lags <= CORR_MAX_LAGS; }
+// The plan's own window length where it has register transforms, else the
+// shortest one whose windows are at least half exact (a quarter at most lags).
+static int corr_fft_len(const Plan* p) {
+  if (reg_log_n1(p->M) > 0) return p->M;
+  int M = 1 << 14;
+  while (M < (1 << 18) && M < 4 * p->n_lags) M <<= 1;
+  return M;
+}
+
+// Transforms or direct sums, by the time that each is expected to take (both
+// measured at 2e3 to 2e7 samples in intervals of 100 to 2e6, 1 to 60000 lags and 1
+// to 2000 filters): a pair of windows takes 17 ps a point, a filter's float64
+// transform 100 ps a point, their launches 60 us; the direct sums 0.245 ns a sample
+// per block of CORR_LB lags, 3.5 ns an item, 6 ps for each atomic it ends with, and
+// at least 38 us for each thousand samples of the longest item.  So windows of 2^14
+// points are not spent on short intervals (2e6 samples, 50 lags, direct against
+// transforms: intervals of 100 0.57 and 2.77 ms, of 300 0.49 and 0.98 ms, of 1000
+// 0.49 and 0.34 ms, of 10000 0.74 and 0.08 ms).
+static bool fft_cheaper(const Plan* p) {
+  if (p->n_lags > CORR_MAX_LAGS) return false;
+  const long long M = corr_fft_len(p), h = p->n_lags - 1, U = M - 2 * h;
+  std::vector<long long> windows(p->n_filters, 0);
+  double samples = 0, items = 0, longest = 0;
+  for (int i = 0; i < p->n_ivl; ++i) {
+    const long long n = p->offsets[i + 1] - p->offsets[i];
+    if (n <= 0) continue;
+    windows[p->ivl_filter[i]] += n + h <= M ? 1 : (n + U - 1) / U;
+    samples += (double)((n + 7) / 8 * 8);
+    items += (double)((n + CORR_CHUNK - 1) / CORR_CHUNK);
+    longest = std::max(longest, (double)std::min<long long>(n, CORR_CHUNK));
+  }
+  double pairs = 0;
+  for (long long w : windows) pairs += (double)((w + 1) / 2);
+  const double blocks = (double)((p->n_lags + CORR_LB - 1) / CORR_LB);
+  const double t_fft = 60.0 + (17e-6 * pairs + 100e-6 * p->n_filters) * M;   // microseconds
+  const double t_direct = std::max(blocks * (0.245e-3 * samples + 3.5e-3 * items) + 6e-6 * items * p->n_lags,
+                                   38e-3 * longest);
+  return t_fft < t_direct;
+}
+
+bool corr_by_fft(Plan* p) {
+  if (p->corr.route == 0) p->corr.route = fft_cheaper(p) ? 1 : 2;
+  return p->corr.route == 1;
+}
 
 madmap_status corr_setup(Plan* p, cudaStream_t s) {
   CorrPlan& c = p->corr;
   if (c.G) return MADMAP_OK;
   madmap_status st = MADMAP_OK;
-  // the plan's own window length where it has register transforms, else the
-  // shortest one whose windows are at least half exact (a quarter at most lags)
-  int M = p->M;
-  const bool own = reg_log_n1(M) == 0;
-  if (own) {
-    M = 1 << 14;
-    while (M < (1 << 18) && M < 4 * p->n_lags) M <<= 1;
-  }
+  const int M = corr_fft_len(p);
+  const bool own = reg_log_n1(p->M) == 0;   // tables of this pass's own
   c.M = M;
   const int rl = reg_log_n1(M), lg = rl + 8;
   c.logN2 = (lg + 1) / 2;

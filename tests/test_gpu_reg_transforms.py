@@ -119,6 +119,36 @@ def test_lag_gradient_matches_direct_correlation(lg):
     assert np.abs(host(gl) - ogl).max() < 4 * TOL * scale, np.abs(host(gl) - ogl).max() / scale
 
 
+@pytest.mark.parametrize("lens, n_filters, transforms", [
+    ((20000, 40000), 1, True),
+    ((100,) * 600, 1, False),          # windows of 2^14 points for 100 samples each
+    ((1000,) * 300, 300, False),       # a float64 transform for each filter's interval
+    ((3000,) * 100, 3, True)])
+def test_lag_gradient_by_the_cheaper_way(lens, n_filters, transforms):
+    """Transforms or direct sums by their expected time: the transforms' buffers (a
+    window pair's 2^15 points or more) show in the plan's device memory; the lags
+    match direct sums in 64 bits within the bound above either way."""
+    import paper_0906_1775_gb300 as mm
+    from oracle.adjoint import solve_backward
+    p = tiny_T(seed=131, n=sum(lens), width=16, n_lags=50, ivls=lens)
+    p.interval_filter = np.arange(len(lens), dtype=np.int32) % n_filters
+    lags = np.repeat(lags_for(p), n_filters, 0)
+    S, plan = system_for(p, lags=lags), make_plan(p, lags=lags)
+    d = cuda(p.d[0])
+    m, _ = plan.solve(d, precision="fp64", rel_tol=1e-12, max_iter=1000)
+    g = np.random.default_rng(2).standard_normal(tuple(m.shape))
+    plan.solve_backward(d, m, cuda(g), precision="fp64", rel_tol=1e-12, max_iter=1000, want_lags=False)
+    before = mm.madmap_plan_get_stats(plan._h)["device_bytes"]
+    _, gl, _ = plan.solve_backward(d, m, cuda(g), precision="fp64", rel_tol=1e-12, max_iter=1000)
+    grown = mm.madmap_plan_get_stats(plan._h)["device_bytes"] - before
+    assert (grown > 8 << 15) == transforms, grown
+    d64 = p.d[0].astype(np.float64)
+    _, ogl, _ = solve_backward(S, d64, host(m), g)
+    lam, _ = S.pcg(g, rel_tol=1e-13, max_iter=2000)
+    scale = np.linalg.norm(S.unpoint(lam)) * np.linalg.norm(d64 - S.unpoint(host(m)))
+    assert np.abs(host(gl) - ogl).max() < 4 * TOL * scale, np.abs(host(gl) - ogl).max() / scale
+
+
 @pytest.mark.parametrize("n_lags", [64, 100, 1024])
 def test_noise_filters_on_the_device_match_the_host(n_lags):
     """set_noise and noise_vjp against madmap_noise_filter and its chain rule: the
