@@ -892,21 +892,26 @@ static int window_align(int n_stokes, int n_lags, int M) {
   return n_stokes == 3 && reg_log_n1(M) > 0 && M - 2LL * (n_lags - 1) >= 64 * WINDOW_ALIGN ? WINDOW_ALIGN : 1;
 }
 
-// align: windows start at multiples of this (window_align).
+// align: windows start at multiples of this (window_align), except in an interval
+// that would need more than a fiftieth more windows for it: one of a window's exact
+// samples or a little less, or of a few times as many, would cost up to twice the
+// transforms for the 1 to 4% that alignment saves.
 static void make_segments(const std::vector<long long>& off, const std::vector<int>& filt, int n_lags, int M,
                           int align, std::vector<Seg>& segs) {
   segs.clear();
-  const long long h = n_lags - 1, A = align;
-  const long long U = M - 2 * h - (A - 1);
-  auto down = [A](long long t) { return t >= 0 ? t / A * A : -((-t + A - 1) / A * A); };
+  const long long h = n_lags - 1, exact = M - 2 * h;
   for (size_t i = 0; i + 1 < off.size(); ++i) {
     const long long t0 = off[i], t1 = off[i + 1], n = t1 - t0;
     if (n <= 0) continue;
-    if (n + h + (A - 1) <= M) {
-      const long long ws = down(t0), o = t0 - ws;
-      segs.push_back({ws, t0, t1, (int)o, (int)(o + n), filt[i]});
+    if (n + h <= M) {
+      const long long o = t0 % align + n <= M ? t0 % align : 0;
+      segs.push_back({t0 - o, t0, t1, (int)o, (int)(o + n), filt[i]});
       continue;
     }
+    const long long least = (n + exact - 1) / exact, aligned = exact - (align - 1);
+    const long long A = aligned > 0 && (n + aligned - 1) / aligned - least <= least / 50 ? align : 1;
+    const long long U = exact - (A - 1);
+    auto down = [A](long long t) { return t >= 0 ? t / A * A : -((-t + A - 1) / A * A); };
     for (long long u0 = t0; u0 < t1; u0 += U) {
       const long long u1 = std::min(t1, u0 + U);
       const long long ws = down(u0 - h), o = u0 - ws;   // h <= o < h + A

@@ -170,3 +170,25 @@ def test_noise_filters_on_the_device_match_the_host(n_lags):
         assert np.allclose(out[k], want, rtol=1e-11, atol=1e-11 * np.abs(want).max())
     with pytest.raises(mm.MadmapError):
         plan.set_noise(100.0, prm * np.array([-1.0, 1.0, 1.0]))
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp64", "df64"])
+def test_alignment_takes_no_more_windows(prec):
+    """IQU windows start at multiples of 16 samples, but not where an interval would then
+    need another window: intervals of one window's most samples, of four and of 60 windows'
+    exact ones, and of an odd length (several aligned windows), at odd offsets."""
+    import torch
+    from synth import make_flat_problem
+    n_lags, M = 301, 1 << 14
+    exact = M - 2 * (n_lags - 1)
+    lens = [M - (n_lags - 1), 4 * exact, 60 * exact, 3 * exact + 777]
+    p = make_flat_problem("align", 180, 48, 1, sum(lens), 3, n_lags, det_angles_deg=[0.0], hwp_step_deg=22.5,
+                          interval_lengths=lambda rng, tot: list(lens), noise=(1.0, 1.0, 1.5))
+    plan, S = make_plan(p, fft_len=M), system_for(p)
+    assert plan.stats["n_segments"] == 1 + 4 + 61 + 4
+    x = np.random.default_rng(3).standard_normal((S.n_obs, 3)).astype(np.float32)
+    x[S.excised] = 0.0
+    y = host(plan.apply_ATNA(cuda(x, torch.float32 if prec == "fp32" else torch.float64), precision=prec))[0]
+    assert rel_rms(y, S.H(x.astype(np.float64))) < 2 * TOLS[prec]
+    b = host(plan.rhs(cuda(p.d), precision=prec))[0]
+    assert rel_rms(b, S.rhs(p.d[0])) < 2 * TOLS[prec]
