@@ -365,8 +365,8 @@ class Plan:
     the ranks, e.g. torch_allreduce().  Every rank must make the same calls.
     deterministic = True sums every map in a fixed order (bit-reproducible maps).
     autotune = True times candidate FFT lengths and launch chunk sizes, then the
-    other split of the length into column and row transforms and the scatter with
-    and without run sums, and keeps the fastest (stats["tuned"] lists
+    other split of a length of 2^19 into column and row transforms and the scatter
+    with and without run sums, and keeps the fastest (stats["tuned"] lists
     (fft_len, tiles_per_chunk, ms, runs, n2) per candidate).
     scatter_runs = 1 / -1 forces the scatter's run sums on / off (0: the plan's rule).
     fft_split = 1 makes the FFT's column transforms half the default length.

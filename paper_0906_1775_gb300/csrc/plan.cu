@@ -1464,7 +1464,7 @@ static constexpr double kRunsMinFrac = 0.25;
 // warm-up application) for every candidate FFT length (the given one, or the
 // cost model's choice and its neighbours a factor two either way) and tiles
 // per launch chunk (the given number, or the default rule and half and twice
-// it); at the fastest of those, the other split of the length into column and
+// it); at the fastest of those, the other split of a length of 2^19 into column and
 // row transforms (columns half as long, rows twice) and then the scatter with
 // and without run sums.  The fastest candidate is kept; all of them are
 // reported in the plan's stats.
@@ -1550,9 +1550,9 @@ static madmap_status autotune_windows(Plan* p, int M_fixed, int M0, long long tp
     *out_ms = ms / 3;
     return r;
   };
-  // the other split of the best length: columns of half the length (kept when
-  // both transforms still have compile-time geometry)
-  if (st == MADMAP_OK && !p->split_fixed) {
+  // the other split of the best length: columns of half the length (where the length
+  // has a split, and both transforms still have compile-time geometry)
+  if (st == MADMAP_OK && !p->split_fixed && reg_log_n1(bestM) == 0) {
     const int lg = ilog2((unsigned)bestM), l2 = (lg + 1) / 2 - 1, l1 = lg - l2;
     if (l2 >= 7 && l2 <= 10 && l1 >= 6 && l1 <= 10) {
       p->split_down = 1;

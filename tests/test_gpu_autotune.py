@@ -33,11 +33,20 @@ def test_autotuned_plan_reports_candidates_and_keeps_the_fastest():
     assert all(ms > 0 for _, _, ms, _, _ in tuned)
     m_best, t_best, _, r_best, n2_best = min(tuned, key=lambda c: c[2])
     assert (st["fft_len"], st["tiles_per_chunk"], st["scatter_runs"], st["n2"]) == (m_best, t_best, r_best, n2_best)
-    # both scatter modes and both column lengths were timed at the chosen length
+    # both scatter modes were timed at the chosen length, and both column lengths where it has two
     assert {r for m, t, _, r, _ in tuned if (m, t) == (m_best, t_best)} == {0, 1}
-    lg = m_best.bit_length() - 1
-    n_splits = 2 if 7 <= (lg + 1) // 2 - 1 and lg - ((lg + 1) // 2 - 1) <= 10 else 1
+    n_splits = 2 if m_best == 1 << 19 else 1
     assert len({n2 for m, t, _, _, n2 in tuned if (m, t) == (m_best, t_best)}) == n_splits
+
+
+@pytest.mark.parametrize("fft_len, splits", [(1 << 15, 1), (1 << 16, 1), (1 << 18, 1), (1 << 19, 2)])
+def test_the_other_split_is_timed_only_where_there_is_one(fft_len, splits):
+    """Lengths of 2^14 to 2^18 run columns of 256 points whatever the split: a second
+    candidate there would time the same kernels twice."""
+    st = make_plan(_problem(), autotune=True, fft_len=fft_len).stats
+    assert len({n2 for _, _, _, _, n2 in st["tuned"]}) == splits
+    if splits == 1:
+        assert st["n2"] == 1 << (fft_len.bit_length() // 2)
 
 
 def test_every_candidate_length_gives_the_exact_product():
@@ -71,7 +80,7 @@ def test_autotuned_plan_operator_and_solve_match_oracle():
     assert rel_rms(host(m), xo) < 1e-10
 
 
-@pytest.mark.parametrize("fft_len", [1 << 13, 1 << 16, 1 << 17])
+@pytest.mark.parametrize("fft_len", [1 << 13, 1 << 16, 1 << 17, 1 << 19])
 def test_shorter_columns_give_the_same_operator(fft_len):
     """fft_split = 1 (columns half the default length, rows twice): N^-1 against
     the Eq. 15 direct sum, A^T N^-1 A and the right-hand side against the oracle."""
