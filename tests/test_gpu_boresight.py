@@ -24,6 +24,12 @@ FP32_OP_TOL = 2e-5
 FP64_MAP_TOL = 1e-10
 MIXED_MAP_TOL = 1e-6
 
+# One CTA a window (0 and 256 here), the shared-memory kernels (2^13, 2^19), the
+# register transforms (2^14 to 2^18; 2^17 and 2^18 with rows of 512 and 1024 points)
+APPLY_LENS = [0, 256, 1 << 13, 1 << 14, 1 << 17]
+RHS_LENS = [0, 1 << 13, 1 << 16, 1 << 18, 1 << 19]
+LONG_LENS = [1 << 13, 1 << 14, 1 << 16]
+
 
 def _problem(kind):
     from synth.boresight import make_boresight_problem
@@ -108,7 +114,7 @@ def test_observed_and_excised_bit_exact(problems, case, gap):
 
 @pytest.mark.parametrize("case", CASES)
 @pytest.mark.parametrize("prec", ["fp64", "df64", "fp32"])
-@pytest.mark.parametrize("fft_len", [0, 256])
+@pytest.mark.parametrize("fft_len", APPLY_LENS)
 def test_apply_ATNA_vs_oracle(problems, case, prec, fft_len):
     import torch
     p = problems[case]
@@ -124,12 +130,37 @@ def test_apply_ATNA_vs_oracle(problems, case, prec, fft_len):
 
 @pytest.mark.parametrize("case", CASES)
 @pytest.mark.parametrize("prec", ["fp64", "df64", "fp32"])
-def test_rhs_vs_oracle(problems, case, prec):
+@pytest.mark.parametrize("fft_len", RHS_LENS)
+def test_rhs_vs_oracle(problems, case, prec, fft_len):
     p = problems[case]
     S = _system(p)
-    plan = _plan(p)
+    plan = _plan(p, fft_len=fft_len)
     b = host(plan.rhs(cuda(p.d), precision=prec))[0]
     assert rel_rms(b, S.rhs(p.d[0])) < (FP32_OP_TOL if prec == "fp32" else FP64_OP_TOL)
+
+
+@pytest.fixture(scope="module", params=[1, 3])
+def long_case(request):
+    """Intervals of several windows (two or three of 2^14 points) at odd offsets."""
+    from synth.boresight import make_boresight_problem
+    p = make_boresight_problem("bl", 37, 32, 3, 40001, 8, request.param, 33, noise=(1.0, 4.0, 1.5), rot_period=9000,
+                               interval_lengths=lambda rng, n: [29001, 7010, 1, 3989])
+    S = _system(p)
+    x = np.random.default_rng(10).standard_normal((S.n_obs, p.n_stokes)).astype(np.float32)
+    x[S.excised] = 0.0
+    return p, x, S.H(x.astype(np.float64)), S.rhs(p.d[0])
+
+
+@pytest.mark.parametrize("prec", ["fp64", "df64", "fp32"])
+@pytest.mark.parametrize("fft_len", LONG_LENS)
+def test_intervals_of_several_windows(long_case, prec, fft_len):
+    import torch
+    p, x, hx, b = long_case
+    plan = _plan(p, fft_len=fft_len)
+    tol = FP32_OP_TOL if prec == "fp32" else FP64_OP_TOL
+    y = host(plan.apply_ATNA(cuda(x, torch.float32 if prec == "fp32" else torch.float64), precision=prec))[0]
+    assert rel_rms(y, hx) < tol
+    assert rel_rms(host(plan.rhs(cuda(p.d), precision=prec))[0], b) < tol
 
 
 @pytest.mark.parametrize("case", CASES)
@@ -194,10 +225,11 @@ def test_same_maps_as_stored_pointing():
 
 
 @pytest.mark.parametrize("prec", ["fp64", "mixed"])
-def test_solve_batched_matches_oracle(problems, prec):
+@pytest.mark.parametrize("fft_len", [0, 1 << 13, 1 << 14])
+def test_solve_batched_matches_oracle(problems, prec, fft_len):
     p = problems["iqu"]
     S = _system(p)
-    plan = _plan(p)
+    plan = _plan(p, fft_len=fft_len)
     rng = np.random.default_rng(8)
     D = np.stack([p.d[0], rng.standard_normal(p.d[0].shape).astype(np.float32)])
     ms, _ = plan.solve_batched(cuda(D), precision=prec, rel_tol=1e-12, max_iter=600, max_outer=20)

@@ -23,6 +23,12 @@ FP64_MAP_TOL = 1e-10
 MIXED_MAP_TOL = 1e-6
 WHITE = np.array([[1.0]])
 
+# One CTA a window (0 and 256 here), the shared-memory kernels (2^13, 2^19), the
+# register transforms (2^14 to 2^18; 2^17 and 2^18 with rows of 512 and 1024 points)
+APPLY_LENS = [0, 256, 1 << 13, 1 << 14, 1 << 17]
+RHS_LENS = [0, 1 << 13, 1 << 16, 1 << 18, 1 << 19]
+LONG_LENS = [1 << 13, 1 << 14, 1 << 16]
+
 
 def _case(kind):
     """(problem, extra_index, n_extra, oracle lags, library lags, d)"""
@@ -107,7 +113,7 @@ def test_layout_and_excision(cases, case):
 
 @pytest.mark.parametrize("case", CASES)
 @pytest.mark.parametrize("prec", ["fp64", "df64", "fp32"])
-@pytest.mark.parametrize("fft_len", [0, 256])
+@pytest.mark.parametrize("fft_len", APPLY_LENS)
 def test_apply_ATNA_vs_oracle(cases, case, prec, fft_len):
     import torch
     c = cases[case]
@@ -124,13 +130,47 @@ def test_apply_ATNA_vs_oracle(cases, case, prec, fft_len):
 
 @pytest.mark.parametrize("case", CASES)
 @pytest.mark.parametrize("prec", ["fp64", "df64", "fp32"])
-def test_rhs_vs_oracle(cases, case, prec):
+@pytest.mark.parametrize("fft_len", RHS_LENS)
+def test_rhs_vs_oracle(cases, case, prec, fft_len):
     c = cases[case]
     E = _system(c)
-    plan = _plan(c)
+    plan = _plan(c, fft_len=fft_len)
     d = c[5]
     b = host(plan.rhs(cuda(d[None, :]), precision=prec))[0]
     assert rel_rms(b, E.rhs(d)) < (FP32_OP_TOL if prec == "fp32" else FP64_OP_TOL)
+
+
+@pytest.fixture(scope="module")
+def long_case():
+    """Extra columns and half-wave-plate groups over intervals of several windows (two of
+    2^14 points, four of 2^13, less than one of 2^16), at offsets that are not multiples of 16."""
+    from synth import make_flat_problem
+    from synth.extended import add_extra_signal, add_hwp_signal, baseline_index, hwp_inputs
+    lens = [29001, 7010, 1, 4003]
+    n = sum(lens)
+    p = make_flat_problem("extlong", 87, 12, 4, n, 3, 33, det_angles_deg=[0.0, 45.0, 90.0, 135.0], hwp_step_deg=22.5,
+                          interval_lengths=lambda rng, tot: list(lens), noise=(1.0, 4.0, 1.5), flag_frac=0.02)
+    ang, tau, grp, ng = hwp_inputs(p.interval_offsets, p.fs, 1.7, np.random.default_rng(14))
+    grp = np.where(np.arange(len(grp)) % 3 == 1, -1, np.arange(len(grp)) % 3).astype(np.int32)
+    d = add_hwp_signal(p.d[0], p.interval_offsets, ang, tau, grp, np.random.default_rng(15).normal(0.0, 0.3, (3, 32)))
+    idx, n_extra = baseline_index(n, 4, 700)
+    d = add_extra_signal(d, idx, np.random.default_rng(16).normal(0.0, 1.0, n_extra))
+    c = (p, idx, n_extra, lags_for(p), lib_lags(p), d, (ang, tau, grp, 3))
+    E = _system(c)
+    x = np.random.default_rng(17).standard_normal((E.n_obs, E.n_s)).astype(np.float32) * E.active()
+    return c, E, x, E.H(x.astype(np.float64)), E.rhs(d)
+
+
+@pytest.mark.parametrize("prec", ["fp64", "df64", "fp32"])
+@pytest.mark.parametrize("fft_len", LONG_LENS)
+def test_intervals_of_several_windows(long_case, prec, fft_len):
+    import torch
+    c, E, x, hx, b = long_case
+    plan = _plan(c, fft_len=fft_len)
+    tol = FP32_OP_TOL if prec == "fp32" else FP64_OP_TOL
+    y = host(plan.apply_ATNA(cuda(x, torch.float32 if prec == "fp32" else torch.float64), precision=prec))[0]
+    assert rel_rms(y * E.active(), hx) < tol
+    assert rel_rms(host(plan.rhs(cuda(c[5][None, :]), precision=prec))[0], b) < tol
 
 
 @pytest.mark.parametrize("case", CASES)
@@ -181,10 +221,11 @@ def test_destriping_recovers_offsets_on_gpu():
 
 
 @pytest.mark.parametrize("prec", ["fp64", "mixed"])
-def test_solve_batched_matches_oracle(cases, prec):
+@pytest.mark.parametrize("fft_len", [0, 1 << 13, 1 << 14])
+def test_solve_batched_matches_oracle(cases, prec, fft_len):
     c = cases["destripe_IQU"]
     E = _system(c)
-    plan = _plan(c)
+    plan = _plan(c, fft_len=fft_len)
     rng = np.random.default_rng(7)
     D = np.stack([c[5], rng.standard_normal(c[5].shape).astype(np.float32)])
     ms, _ = plan.solve_batched(cuda(D), precision=prec, rel_tol=1e-12, max_iter=3000, max_outer=30)

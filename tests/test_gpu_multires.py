@@ -21,6 +21,12 @@ FP32_OP_TOL = 2e-5
 FP64_MAP_TOL = 1e-10
 MIXED_MAP_TOL = 1e-6
 
+# One CTA a window (0 and 256 here), the shared-memory kernels (2^13, 2^19), the
+# register transforms (2^14 to 2^18; 2^17 and 2^18 with rows of 512 and 1024 points)
+APPLY_LENS = [0, 256, 1 << 13, 1 << 14, 1 << 17]
+RHS_LENS = [0, 1 << 13, 1 << 16, 1 << 18, 1 << 19]
+LONG_LENS = [1 << 13, 1 << 14, 1 << 16]
+
 
 def _problem(seed=5, noiseless=False, width=8, factor=2, n=600, n_lags=10, lo=80, hi=300, flag_frac=0.0):
     from synth import make_flat_problem
@@ -94,7 +100,7 @@ def test_indexing_and_excision_bit_exact(case, kind):
 @pytest.mark.parametrize("case", list(CASES))
 @pytest.mark.parametrize("kind", ["plain", "planted"])
 @pytest.mark.parametrize("prec", ["fp64", "df64", "fp32"])
-@pytest.mark.parametrize("fft_len", [0, 256])
+@pytest.mark.parametrize("fft_len", APPLY_LENS)
 def test_apply_ATNA_vs_oracle(case, kind, prec, fft_len):
     import torch
     p = CASES[case]()
@@ -109,12 +115,34 @@ def test_apply_ATNA_vs_oracle(case, kind, prec, fft_len):
 
 @pytest.mark.parametrize("case", list(CASES))
 @pytest.mark.parametrize("prec", ["fp64", "df64", "fp32"])
-def test_rhs_vs_oracle(case, prec):
+@pytest.mark.parametrize("fft_len", RHS_LENS)
+def test_rhs_vs_oracle(case, prec, fft_len):
     p = CASES[case]()
     M = _system(p, "planted")
-    plan = _plan(p, "planted")
+    plan = _plan(p, "planted", fft_len=fft_len)
     b = host(plan.rhs(cuda(p.d), precision=prec))[0]
     assert rel_rms(b, M.rhs(p.d[0])) < (FP32_OP_TOL if prec == "fp32" else FP64_OP_TOL)
+
+
+@pytest.fixture(scope="module")
+def long_case():
+    """Intervals of several windows (two or three of 2^14 points), some ending in a window's first samples."""
+    p = _problem(seed=15, n=40001, n_lags=33, lo=3000, hi=35000, flag_frac=0.02)
+    M = _system(p, "planted")
+    x = np.random.default_rng(13).standard_normal((M.n_obs, 3)).astype(np.float32)
+    return p, x, M.H(x.astype(np.float64)), M.rhs(p.d[0])
+
+
+@pytest.mark.parametrize("prec", ["fp64", "df64", "fp32"])
+@pytest.mark.parametrize("fft_len", LONG_LENS)
+def test_intervals_of_several_windows(long_case, prec, fft_len):
+    import torch
+    p, x, hx, b = long_case
+    plan = _plan(p, "planted", fft_len=fft_len)
+    tol = FP32_OP_TOL if prec == "fp32" else FP64_OP_TOL
+    y = host(plan.apply_ATNA(cuda(x, torch.float32 if prec == "fp32" else torch.float64), precision=prec))[0]
+    assert rel_rms(y, hx) < tol
+    assert rel_rms(host(plan.rhs(cuda(p.d), precision=prec))[0], b) < tol
 
 
 def test_same_pixelisation_equals_single_resolution_plan():
@@ -180,10 +208,11 @@ def test_noiseless_recovery_on_gpu():
 
 
 @pytest.mark.parametrize("prec", ["fp64", "mixed"])
-def test_solve_batched_matches_single_solves(prec):
+@pytest.mark.parametrize("fft_len", [0, 1 << 13, 1 << 14])
+def test_solve_batched_matches_single_solves(prec, fft_len):
     p = CASES["small"]()
     M = _system(p, "planted")
-    plan = _plan(p, "planted")
+    plan = _plan(p, "planted", fft_len=fft_len)
     rng = np.random.default_rng(5)
     D = np.stack([p.d[0], p.d[0] * 0.5 + rng.standard_normal(p.d[0].shape).astype(np.float32),
                   rng.standard_normal(p.d[0].shape).astype(np.float32)])

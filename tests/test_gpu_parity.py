@@ -251,14 +251,16 @@ def test_iteration_drivers_agree(prec):
         assert rel_rms(host(m), host(runs[0][0])) < (1e-12 if prec == "fp64" else 1e-9)
 
 
-def test_chunks_on_two_streams_match_one_launch():
+@pytest.mark.parametrize("fft_len", [256, 1 << 13, 1 << 14])
+def test_chunks_on_two_streams_match_one_launch(fft_len):
     """Several chunks per application run on two plan streams (inside the solver's
-    graphs too); operator and solves agree with the one-launch plan and the oracle."""
+    graphs too); operator and solves agree with the one-launch plan and the oracle, for
+    one CTA a window, the shared-memory kernels and the register transforms."""
     torch = _torch()
     p = tiny_IQU(seed=23, n_per_det=2000, n_ivl_lo=100, n_ivl_hi=900)
     S = system_for(p)
-    one = make_plan(p, fft_len=256)
-    many = make_plan(p, fft_len=256, tiles_per_chunk=2)
+    one = make_plan(p, fft_len=fft_len)
+    many = make_plan(p, fft_len=fft_len, tiles_per_chunk=2)
     assert many.stats["n_tiles"] >= 8 and many.stats["tiles_per_chunk"] == 2
     x = np.random.default_rng(2).standard_normal((S.n_obs, 3))
     ref = S.H(x)

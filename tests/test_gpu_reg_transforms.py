@@ -181,11 +181,11 @@ def test_alignment_takes_no_more_windows(prec):
     from synth import make_flat_problem
     n_lags, M = 301, 1 << 14
     exact = M - 2 * (n_lags - 1)
-    lens = [M - (n_lags - 1), 4 * exact, 60 * exact, 3 * exact + 777]
+    lens = [3 * exact + 777, M - (n_lags - 1), 4 * exact, 60 * exact]
     p = make_flat_problem("align", 180, 48, 1, sum(lens), 3, n_lags, det_angles_deg=[0.0], hwp_step_deg=22.5,
                           interval_lengths=lambda rng, tot: list(lens), noise=(1.0, 1.0, 1.5))
     plan, S = make_plan(p, fft_len=M), system_for(p)
-    assert plan.stats["n_segments"] == 1 + 4 + 61 + 4
+    assert plan.stats["n_segments"] == 4 + 1 + 4 + 61
     x = np.random.default_rng(3).standard_normal((S.n_obs, 3)).astype(np.float32)
     x[S.excised] = 0.0
     y = host(plan.apply_ATNA(cuda(x, torch.float32 if prec == "fp32" else torch.float64), precision=prec))[0]

@@ -98,6 +98,25 @@ def test_noalloc_weighting_several_chunks_allocates_nothing():
     assert rel_rms(host(w), ref) < TOL["fp64"]
 
 
+@pytest.mark.parametrize("n_lags", [3000, 1 << 13, 12345, 1 << 15])
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+def test_noalloc_weighting_at_each_long_window(n_lags, prec):
+    """Windows of 2^14 to 2^17 points: in float32 the register transforms, whose tables
+    stand where the other kernels' twiddles do."""
+    import torch
+    from oracle.noise import apply_ninv_fft
+    n = 400_003
+    off = np.array([0, 1, 1 + 3 * n_lags, n], dtype=np.int64)
+    filt = np.array([0, 1, 1], dtype=np.int32)
+    lags = dominant_lags(2, n_lags, seed=29)
+    yh = np.random.default_rng(12).standard_normal(n).astype(np.float32).astype(np.float64)
+    y = cuda(yh, torch.float64 if prec == "fp64" else torch.float32)
+    w = torch.full_like(y, float("nan"))
+    _noalloc(prec, n, off, filt, lags, y, w)
+    torch.cuda.synchronize()
+    assert rel_rms(host(w), apply_ninv_fft(yh, off, filt, lags, 1 << 18)) < TOL[prec]
+
+
 def test_noalloc_weighting_refuses_stream_capture():
     import torch
     import paper_0906_1775_gb300 as mm
