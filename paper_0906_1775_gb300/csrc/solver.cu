@@ -10,7 +10,7 @@
 //                   residual, best iterate, termination
 //   k_cg_direction  copy x to the best iterate if it improved, p = z + beta p,
 //                   q = 0
-// (maps of up to 16384 rows: k_cg_step does all three in one cluster).
+// (small maps: k_cg_step does all three in one cluster, see cg_step_threads).
 // Dot products are accumulated in float64 in every precision, per block, and
 // the last block to finish (atomic ticket, no waiting) reduces the partials in
 // a fixed order, so results are reproducible run to run.  All scalars live on
@@ -506,7 +506,7 @@ __global__ void __launch_bounds__(NT) k_cg_direction(const Real* x, const Real* 
   }
 }
 
-// One whole iteration after the operator for maps of at most CG_STEP_ROWS rows:
+// One whole iteration after the operator for the maps of cg_step_threads:
 // k_cg_alpha, k_cg_update and k_cg_direction in one cluster of 8 CTAs, the
 // iteration's vectors in registers between the sums and the sums through
 // distributed shared memory (every CTA adds the eight partials in rank order).
@@ -519,7 +519,25 @@ __global__ void __launch_bounds__(NT) k_cg_direction(const Real* x, const Real* 
 // move the vectors slower than 152.
 constexpr int CG_CTAS = 8, CG_ROWS = 4;
 constexpr int CG_THREADS_S = 128, CG_THREADS_L = 512;
-constexpr int CG_STEP_ROWS = CG_CTAS * CG_THREADS_L * CG_ROWS;
+
+// Threads a CTA of k_cg_step for n_rhs maps of n rows, or 0 for the three kernels.
+// 128 up to 4096 rows.  512 above, for temperature only, up to 16384 rows: an IQU row
+// is three times the data, so that the wider CTAs have one SM each and 8 SMs are too
+// few.  With more than 8 right-hand sides only where most of the 512 threads have
+// their rows, since the clusters then queue for the SMs.  Microseconds per iteration
+// (operator included), this kernel and the three, float64 and mixed:
+//   T    4096 rows  38 46, 19 28    64 maps 178 197, 46 65
+//        8192       42 48, 24 30    64 maps 378 370, 119 112
+//       16384       45 48, 27 30    64 maps 688 699, 194 202
+//   IQU  4096       47 53, 25 32    8 maps  69 76, 28 35
+//        8192       57 55, 34 33    16 maps 239 229, 81 73
+//       16384       93 81, 48 37    16 maps 438 423, 124 108
+template <int NS>
+static int cg_step_threads(int n, int n_rhs) {
+  if (n <= CG_CTAS * CG_THREADS_S * CG_ROWS) return CG_THREADS_S;
+  constexpr int most = CG_CTAS * CG_THREADS_L * CG_ROWS;
+  return NS == 1 && n <= most && (n_rhs <= 8 || n > most / 4 * 3) ? CG_THREADS_L : 0;
+}
 
 // The cluster's sum of v in thread 0 of every CTA (part: this CTA's list of the
 // CTAs' sums, warp: its warps').
@@ -870,16 +888,20 @@ static void enqueue_iteration(Plan* p, SolveBuffers* sb, const Batch& B, cudaStr
   // sharded plans: q = sum over the ranks of their shares of H p
   if (*st == MADMAP_OK)
     *st = reduce_across(p, q, nv * B.n_rhs, sizeof(Real) == 8 ? MADMAP_REDUCE_F64 : MADMAP_REDUCE_F32, s);
-  if (n <= CG_STEP_ROWS) {
-    count_launches(1);
-    const dim3 gs(CG_CTAS, B.n_rhs);
-    if (n <= CG_CTAS * CG_THREADS_S * CG_ROWS)
-      k_cg_step<Real, NS, CG_THREADS_S><<<gs, CG_THREADS_S, 0, s>>>(x, r, z, pp, q, xb, nv, n, p->P64, p->P32,
-                                                                    p->fp64flag, sb->st, sb->hist);
-    else
+  const int threads = cg_step_threads<NS>(n, B.n_rhs);
+  const dim3 gs(CG_CTAS, B.n_rhs);
+  if (threads > 0) count_launches(1);
+  if (threads == CG_THREADS_S) {
+    k_cg_step<Real, NS, CG_THREADS_S><<<gs, CG_THREADS_S, 0, s>>>(x, r, z, pp, q, xb, nv, n, p->P64, p->P32,
+                                                                  p->fp64flag, sb->st, sb->hist);
+    return;
+  }
+  if constexpr (NS == 1) {
+    if (threads == CG_THREADS_L) {
       k_cg_step<Real, NS, CG_THREADS_L><<<gs, CG_THREADS_L, 0, s>>>(x, r, z, pp, q, xb, nv, n, p->P64, p->P32,
                                                                     p->fp64flag, sb->st, sb->hist);
-    return;
+      return;
+    }
   }
   count_launches(3);
   k_cg_alpha<Real, NS><<<g, NT, 0, s>>>(pp, q, nv, n, sb->st, sb->partials);

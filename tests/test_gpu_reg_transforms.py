@@ -92,6 +92,45 @@ def test_solve_around_the_cluster_kernel_s_map_sizes(width, prec):
     assert rel_rms(host(two[1]), 2 * x) < 1e-9 and infos[0]["status"] == 0
 
 
+@pytest.mark.parametrize("stokes, rows, n_rhs, launches", [
+    (1, 4096, 1, 1), (1, 4097, 1, 1), (1, 16384, 1, 1), (1, 16385, 1, 3),
+    (1, 4096, 9, 1), (1, 4097, 8, 1), (1, 4097, 9, 3), (1, 12288, 9, 3), (1, 12289, 9, 1),
+    (3, 4096, 1, 1), (3, 4096, 9, 1), (3, 4097, 1, 3), (3, 16384, 1, 3)])
+def test_vector_kernels_of_an_iteration_by_map_and_batch_size(stokes, rows, n_rhs, launches):
+    """Which maps run the cluster kernel (its one launch an iteration or the three of the
+    vector kernels, beside the operator's own), and that both reach the map."""
+    import torch
+    import paper_0906_1775_gb300 as mm
+    rng = np.random.default_rng(rows + stokes)
+    pix = np.concatenate([np.arange(rows), rng.permutation(rows), rng.permutation(rows), np.arange(rows)]).astype(np.int32)
+    n = pix.size
+    psi = np.repeat([0.0, 0.8, 1.6, 2.4], rows).astype(np.float32) if stokes == 3 else None
+    lags = np.array([[1.0, 0.2, 0.05]])
+    plan = mm.Plan(cuda(pix), cuda(psi) if stokes == 3 else None, rows, [0, n], [0], lags, fft_len=1024,
+                   tiles_per_chunk=100000)
+    assert plan.n_obs == rows and plan.stats["n_excised"] == 0
+    d = rng.standard_normal(n).astype(np.float32)
+    D = cuda(np.stack([2.0 ** (k % 4) * d for k in range(n_rhs)]).astype(np.float32))
+    from oracle.solver import System
+    S = System(pix, psi, rows, stokes, np.array([0, n]), np.array([0]), lags)
+    x, _ = S.solve(d, rel_tol=1e-13, max_iter=200)
+
+    def solve(iters):
+        kw = dict(precision="fp64", rel_tol=0.0, max_iter=iters, use_graph=0, iters_per_sync=1)
+        torch.cuda.synchronize()
+        before = mm.madmap_kernel_launch_count()
+        m = plan.solve(D[0], **kw)[0][None] if n_rhs == 1 else plan.solve_batched(D, **kw)[0]
+        return mm.madmap_kernel_launch_count() - before, host(m)
+
+    solve(1)
+    # the operator: one launch a chunk of tiles, two windows or right-hand sides a tile
+    st = plan.stats
+    chunks = -(-(-(-st["n_segments"] * n_rhs // 2)) // st["tiles_per_chunk"])
+    assert solve(4)[0] - solve(2)[0] == 2 * (chunks + launches)
+    for k, m in enumerate(solve(30)[1]):
+        assert rel_rms(m, 2.0 ** (k % 4) * x) < 1e-9
+
+
 @pytest.mark.parametrize("lg", [13, 14, 15, 16, 17, 18, 19])
 def test_lag_gradient_matches_direct_correlation(lg):
     """The backward pass's lag correlation by windowed transforms, on intervals
