@@ -516,13 +516,14 @@ madmap_status madmap_polarisation_weights(int32_t precision, int64_t n, const fl
                                           void* sin2psi, void* stream);
 
 /* Times the operator H = A^T N^-1 A in the plan's launch configuration:
- * `reps` applications to the plan's current search-direction buffer.  First
- * with CUDA events recorded on `stream` around every launch of each of the
+ * `reps` applications to the plan's current search-direction buffer, after one
+ * that is not timed.  First with CUDA events recorded on `stream` around every launch of each of the
  * three operator kernels (gather + column FFTs; row FFTs x filter spectrum;
  * inverse column FFTs + scatter), the chunks run one after another; then
  * `reps` applications as the solver launches them (chunks of one application
  * overlapped on two plan streams) between two events on `stream`.
- * ms_out (host [4]): [0..2] mean duration of one launch of each kernel, [3]
+ * ms_out (host [4]): [0..2] mean duration of one launch of each kernel (where one
+ * kernel does the work: it, then zeros), [3]
  * mean duration of one application.  launches_out (host [3], may be NULL):
  * launches of each kernel per application.  Synchronises `stream`.
  * precision: FP64, FP32 or DF64. */

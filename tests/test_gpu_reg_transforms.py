@@ -231,3 +231,24 @@ def test_alignment_takes_no_more_windows(prec):
     assert rel_rms(y, S.H(x.astype(np.float64))) < 2 * TOLS[prec]
     b = host(plan.rhs(cuda(p.d), precision=prec))[0]
     assert rel_rms(b, S.rhs(p.d[0])) < 2 * TOLS[prec]
+
+
+@pytest.mark.parametrize("fft_len", [1 << 11, 1 << 13, 1 << 15])
+def test_operator_timing_leaves_the_kernels_loading_out(fft_len):
+    """In a fresh process the first launch of a kernel loads it, which takes milliseconds
+    where the kernels take tens of microseconds: the first timing agrees with the second."""
+    import os
+    import subprocess
+    import sys
+    code = f"""
+from tests.gpu_helpers import make_plan
+from tests.helpers import tiny_IQU
+plan = make_plan(tiny_IQU(seed=190, n_per_det=20000, n_lags=40, n_ivl_lo=2000, n_ivl_hi=9000), fft_len={fft_len})
+for prec in ("fp32", "fp64", "df64"):
+    first, second = (plan.time_operator(prec, reps=2)[0] for _ in range(2))
+    assert 0 < sum(first[:3]) < 5 * sum(second[:3]), (prec, first, second)
+print("DONE")
+"""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    out = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, cwd=root, timeout=300)
+    assert "DONE" in out.stdout, out.stdout + out.stderr
