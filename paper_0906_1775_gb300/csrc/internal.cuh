@@ -745,8 +745,33 @@ constexpr int OP_THREADS = 256;
 // its twiddles, and the most that one CTA takes (k_one; two CTAs per SM).
 inline size_t one_smem(int esz, int lg) { return (size_t)(lay_rs(esz, lg, false) + (1 << lg)) * esz; }
 constexpr size_t ONE_SMEM = (size_t)100 << 10;
-inline bool one_cta(const Plan* p, int esz) {
+inline bool one_fits(const Plan* p, int esz) {
   return p->reg.logN1 == 0 && one_smem(esz, p->logN1 + p->logN2) <= ONE_SMEM;
+}
+// Whether k_one also runs an application of n_tiles tiles: on a few waves of CTAs it
+// always saves launches and the trips through scratch, on many its two CTAs an SM hide
+// less latency than the four of k_f1 and k_f3, which shows where a sample costs most
+// beside its transform (k_one and the three kernels, us):
+//   float32, half-wave-plate terms: 4 x 2^19 samples at M = 2048 102 102, 4 x 2^20 242
+//     204 (right-hand side 189 140), 4 x 2^22 912 736;
+//   float32, other extended IQU pointing from M = 1024 on: 4 x 2^20 samples at M = 2048
+//     95 99, 4 x 3 2^19 144 139, 4 x 2^21 191 177 (right-hand side 156 141);
+//   float32 gathers of on-the-fly pointing from M = 2048 on: 99 104, 141 138, 175 164.
+// Stored pointing and the shorter windows gain at every size (IQU, 4 x 2^22 samples:
+// M = 512 359 413, M = 4096 212 229).  Float64 at M = 256 lasts as long as the SM with
+// the most tiles, four at a time: 460 tiles 38 44, 610 52 46, 9620 497 462.
+enum { WORK_PLAIN = 0, WORK_OTF = 1, WORK_EXT = 2, WORK_HWP = 3 };
+inline bool one_cta(const Plan* p, int prec, int work, int n_tiles) {
+  if (!one_fits(p, prec == OPP_F32 ? sizeof(float2) : sizeof(double2))) return false;
+  if (prec == OPP_F64) return p->M > 256 || n_tiles <= 4 * 152;
+  if (prec == OPP_DF64 || work == WORK_PLAIN) return true;
+  const long long points = (long long)n_tiles * p->M;
+  if (work == WORK_HWP) return points <= 3LL << 19;
+  return p->M < (work == WORK_EXT ? 1024 : 2048) || points <= 3LL << 20;
+}
+// of the map-to-map operator
+inline int operator_work(const Plan* p) {
+  return p->hwp_base ? WORK_HWP : p->ext && p->n_stokes == 3 ? WORK_EXT : p->otf ? WORK_OTF : WORK_PLAIN;
 }
 // Tiles of one launch of a tile set where scratch allows: at least two launches
 // from 16 tiles on, so that the two streams overlap.

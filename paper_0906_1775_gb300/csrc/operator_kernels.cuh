@@ -24,6 +24,7 @@
 // inverses consume it, so no reordering pass exists anywhere.
 #pragma once
 
+#include <limits.h>
 #include <math.h>
 
 #include <algorithm>
@@ -1680,7 +1681,11 @@ madmap_status launch_all(Plan* p, const void* in, void* out, long long in_stride
   const int n_tiles = ts ? ts->n_tiles : p->n_tiles;
   const bool reg = p->reg.logN1 > 0;   // register transforms
   const size_t sm1 = one_smem(sizeof(typename CxT<Real>::type), p->logN1 + p->logN2);
-  const bool one = one_cta(p, sizeof(typename CxT<Real>::type));   // a tile per CTA
+  constexpr int prec = DF ? OPP_DF64 : sizeof(Real) == 8 ? OPP_F64 : OPP_F32;
+  const int work = OUT != OUT_MAP ? WORK_PLAIN
+                   : extended(NS) ? (p->hwp_base ? WORK_HWP : NS == NS_EXT_IQU ? WORK_EXT : WORK_PLAIN)
+                   : on_the_fly(NS) && gathers(IN) ? WORK_OTF : WORK_PLAIN;
+  const bool one = one_cta(p, prec, work, n_tiles);   // a tile per CTA
   const size_t sm13 = smem_f13<Real>(p), sm2 = smem_f2<Real>(p);
   const OpKernels K = pick_kernels<Real, NS, IN, OUT>(p);
   a.reg_logN1 = p->reg.logN1;
@@ -1690,13 +1695,15 @@ madmap_status launch_all(Plan* p, const void* in, void* out, long long in_stride
   a.reg_four0 = p->reg.four0;
   a.reg_wide = DF ? (const void*)p->wide_df : (const void*)p->wide64;
   // n_rhs == 0 only sets the kernels' attributes, so it can precede a capture
-  if (one) {
-    MM_CUDA(set_smem(k_one<Real, NS, IN, OUT>, sm1));
-  } else if (!reg) {
+  // (of both ways of short windows where a tile set may take the other one)
+  const bool ahead = n_rhs == 0;
+  if (one || (ahead && one_cta(p, prec, work, 1))) MM_CUDA(set_smem(k_one<Real, NS, IN, OUT>, sm1));
+  if (!reg && (!one || (ahead && !one_cta(p, prec, work, INT_MAX)))) {
     MM_CUDA(set_smem(K.f1, sm13));
     MM_CUDA(set_smem(K.f3, sm13));
     MM_CUDA(set_smem(K.f2, sm2));
-  } else if (sizeof(Real) == 8 && p->reg.logN1 >= 9) {
+  }
+  if (sizeof(Real) == 8 && p->reg.logN1 >= 9) {
     OpKernel f2;
     int b2;
     size_t sm;

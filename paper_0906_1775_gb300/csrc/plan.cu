@@ -1016,7 +1016,9 @@ static void ensure_batch_scratch(Plan* p, int n_tiles) {
     cudaGetLastError();
     return;
   }
-  if (one_cta(p, sizeof(float2)) && one_cta(p, sizeof(double2))) return;   // no scratch
+  const int work = operator_work(p);
+  if (one_cta(p, OPP_F32, work, n_tiles) && one_cta(p, OPP_F64, work, n_tiles) && one_cta(p, OPP_DF64, work, n_tiles))
+    return;   // no scratch
   const size_t tile = (size_t)p->M * sizeof(double2);
   const size_t want = std::min((size_t)set_chunk(n_tiles) * tile, std::max(tile, BATCH_SLOT_BYTES / tile * tile));
   if (want <= p->batch_slot || (p->scratch_slots > 1 && want <= (size_t)p->tiles_per_chunk * tile)) return;
