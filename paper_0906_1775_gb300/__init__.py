@@ -326,8 +326,9 @@ def madmap_polarisation_weights(psi, precision="fp32", stream=None):
 
 
 def madmap_time_operator(h, precision, reps, stream=None):
-    """(ms[4], launches[3]): mean ms per launch of k_f1, k_f2, k_f3 (chunks in sequence) and, in
-    ms[3], mean ms of one application as solves launch it (chunks overlapped)."""
+    """(ms[4], launches[3]): mean ms per launch of the operator's three kernels (chunks in sequence; where
+    one kernel does the work, it is the first and the others have no launches) and, in ms[3], mean ms of
+    one application as solves launch it (chunks overlapped)."""
     ms = np.zeros(4)
     n = np.zeros(3, dtype=np.int32)
     check(load().madmap_time_operator(h, precision, int(reps), ms.ctypes.data, n.ctypes.data,

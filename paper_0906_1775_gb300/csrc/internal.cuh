@@ -58,7 +58,10 @@ struct DiagItem {
 // kernels' CTAs (152 SMs x 4 CTAs x 4096 elements) at 16 bytes an element.  A
 // set has its own chunks instead of the plan's, which are sized for one right-hand
 // side (16 right-hand sides of 2.5e6 samples, M = 2^16: 31 launches of 208 CTAs
-// for 608 resident ones); smaller sets take what half of their tiles need.
+// for 608 resident ones; a mixed solve at 1, 20, 40, 80 and 159 MB a slot: 9.9, 7.5,
+// 7.4, 7.9 and 7.5 ms, of 16 IQU right-hand sides of 2^22 samples 26.4, 26.4, 24.2,
+// 23.3 and 22.1 ms, and 2 to 8 right-hand sides alike); smaller sets take what half
+// of their tiles need.
 constexpr size_t BATCH_SLOT_BYTES = (size_t)4 * 152 * 4 * 4096 * 16;
 
 // A list of tiles whose lanes name their right-hand side (batched solves).

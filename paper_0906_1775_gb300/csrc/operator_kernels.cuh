@@ -110,7 +110,7 @@ struct OpArgs {
   int reg_logN1;
   const float4 *reg_col, *reg_row, *reg_four;
   const float2* reg_four0;
-  const void* reg_wide;  // the float64-size types' (WideTables)
+  const void* reg_wide;  // the float64-size types' (wide_four in internal.cuh)
   int n_rep;          // > 1: map outputs go to replica (blockIdx.x + blockIdx.y) % n_rep, rep_stride apart
   int runs;           // scatter runs of consecutive samples that hit one pixel with one atomic (run_*)
   long long rep_stride;
@@ -1151,7 +1151,7 @@ __global__ void __launch_bounds__(256, sizeof(Real) == 4 ? MM_MINB_F13 : MM_MINB
 }
 
 
-// Lanes of a run sum (run_sum): a run of samples in one pixel adds once per
+// Lanes of a run sum (run_sums): a run of samples in one pixel adds once per
 // aligned group of this many, here the 16 consecutive samples of a warp's row.
 // Shorter groups take fewer shuffles (a third of k_c3's L1 wavefronts on the ring
 // scan, 0.65 repeats: 16, 8 and 4 lanes take 103.5, 97.9 and 97.6 us per launch,

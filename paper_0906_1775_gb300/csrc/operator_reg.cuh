@@ -164,7 +164,7 @@ __host__ __device__ constexpr int reg_batch() {
 }
 
 // Twiddles of the float64-size types, read whole (a product costs more than
-// the read): entries of the plan's WideTables, or of the float32 powers.
+// the read): entries of the plan's wide tables (wide_four), or of the float32 powers.
 template <typename Real>
 struct ColTwiddle {   // w^m = exp(-2 pi i j m / 256)
   typedef typename CxT<Real>::type C;
@@ -501,9 +501,10 @@ inline madmap_status launch_rows(OpArgs a, int nt, cudaStream_t s) {
 // Float64 on the smallest problems: with fewer than two column CTAs per SM the
 // launch lasts as long as the SM with the most of them, whose float64 pipe every
 // CTA waits for, so both column kernels run 2 columns and the rows one warp a CTA
-// (1024 columns and 6 tiles of 2^15: 96 CTAs on 152 SMs become 384; one
-// application 75.5 -> 70.2 us, a solve 1.61 -> 1.52 ms; the line at 1, 4 or 8
-// CTAs per SM measures the same there, larger problems lose coalescing).
+// (one application, wide against narrow CTAs, at 16, 96, 176 and 344 wide CTAs a
+// launch: temperature 62.7 and 56.7, 79.2 and 76.2, 134.8 and 109.1, 258 and 265 us;
+// IQU 76.3 and 69.5, 93.6 and 87.5, 149 and 124, 286 and 301 us; from 350 on, 1 to
+// 5% the other way, for coalescing).
 template <typename Real, int NS>
 constexpr bool narrow_ctas() {
   return std::is_same<Real, double>::value && (NS == 1 || NS == 3);

@@ -191,7 +191,7 @@ __global__ void k_fill_twiddles(double2* tw, int M) {
   }
 }
 
-// WideTables of length M = 256 N1 from the table of M-th roots.
+// The wide tables (wide_four) of length M = 256 N1 from the table of M-th roots.
 template <typename C>
 __global__ void k_wide_tables(const C* tw, C* out, int logN1) {
   const int N1 = 1 << logN1, M = N1 << 8, lb = wide_lb(logN1), la = logN1 - lb, n = wide_four(logN1) + M;
